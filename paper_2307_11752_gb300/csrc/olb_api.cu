@@ -263,6 +263,15 @@ int olb::device_sm_count() {
   return n;
 }
 
+int64_t olb::device_l2_bytes() {
+  int dev = 0, n = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrL2CacheSize, dev) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return n;
+}
+
 bool olb::encode_population_map(void* map, int elem_bytes, bool bf16, const void* base, int nx, int ny, int nz,
                                 int q, int pitch, int box_x, int box_rows) {
   static PFN_cuTensorMapEncodeTiled_v12000 encode = nullptr;
@@ -312,6 +321,8 @@ int olb::set_error(int code, const char* msg) {
 // ---------------------------------------------------------------------------------
 struct olb_lattice {
   int device = 0;  // the CUDA device the handle's buffers live on
+  int sms = 1;     // its SM count
+  int64_t l2_bytes = 0;  // and the size of its L2
   int desc = 0, dtype = 0, q = 0, dim = 0;
   int nx = 0, ny = 0, nz = 0, ncell = 0, pitch = 0;
   const KernelTable* kt = nullptr;
@@ -376,6 +387,9 @@ struct olb_lattice {
     p.err = static_cast<unsigned*>(err.p);
     p.inject_extra_tx = inject_tx;
     p.inject_wait_ns = (unsigned long long)inject_ns;
+    p.device = device;
+    p.sms = sms;
+    p.l2_bytes = l2_bytes;
     p.stream = stream;
     return p;
   }
@@ -577,6 +591,28 @@ int step_once(olb_handle h, bool stats, double* partials, int64_t* rows = nullpt
   return OLB_OK;
 }
 
+// n steps in the handle's scheme without statistics: pairs of pull steps in one pass
+// where the lattice allows it, else step by step.
+int step_many(olb_handle h, int64_t n) {
+  int rc;
+  while (n > 0) {
+    if (n >= 2 && h->scheme == OLB_PULL && h->repr == POST && !h->inject_tx) {
+      const HostParams p = h->params();
+      if (h->kt->step2_ok(p)) {
+        if ((rc = ensure_other(h))) return rc;
+        if ((rc = launched(h, h->kt->step2(p, h->buf[h->cur].p, h->buf[1 - h->cur].p), "step pair"))) return rc;
+        h->cur = 1 - h->cur;
+        h->time += 2;
+        n -= 2;
+        continue;
+      }
+    }
+    if ((rc = step_once(h, false, nullptr))) return rc;
+    --n;
+  }
+  return OLB_OK;
+}
+
 // Reads and clears the handle's error word (synchronises the stream).
 int check_error_word(olb_handle h) {
   unsigned v = 0;
@@ -674,11 +710,10 @@ int adjoint_sweep(olb_handle h, int64_t n_steps, int64_t K, Seed&& seed, double 
     OLB_CUDA(cudaMemcpyAsync(ckpt[s].p, h->buf[h->cur].p, sb, cudaMemcpyDeviceToDevice, h->stream), "checkpoint");
     ckpt_repr[s] = h->repr;
     const int64_t ks = std::min<int64_t>(K, n_steps - s * K);
-    for (int64_t k = 0; k < ks; ++k)
-      if ((rc = step_once(h, false, nullptr))) {
-        h->scheme = saved_scheme;
-        return rc;
-      }
+    if ((rc = step_many(h, ks))) {
+      h->scheme = saved_scheme;
+      return rc;
+    }
   }
   h->scheme = saved_scheme;
 
@@ -783,6 +818,8 @@ int olb_lattice_create(olb_descriptor d, int nx, int ny, int nz, olb_dtype t, ol
   }
   olb_lattice* h = new olb_lattice();
   h->device = device;
+  h->sms = std::max(1, device_sm_count());
+  h->l2_bytes = device_l2_bytes();
   h->desc = (int)d;
   h->dtype = (int)t;
   h->kt = kt;
@@ -1096,9 +1133,7 @@ int olb_step(olb_handle h, int64_t n) {
   int rc = check(h);
   if (rc) return rc;
   if (n < 0) return fail(OLB_ERR_ARG, "negative step count");
-  for (int64_t s = 0; s < n; ++s)
-    if ((rc = step_once(h, false, nullptr))) return rc;
-  return OLB_OK;
+  return step_many(h, n);
 }
 
 int olb_step_stats(olb_handle h, int64_t n, double* out) {
@@ -1107,8 +1142,7 @@ int olb_step_stats(olb_handle h, int64_t n, double* out) {
   if (n < 1) return fail(OLB_ERR_ARG, "olb_step_stats needs n >= 1");
   if (!out) return fail(OLB_ERR_ARG, "null output");
   if ((rc = ensure_partials(h, h->step_rows()))) return rc;
-  for (int64_t s = 0; s + 1 < n; ++s)
-    if ((rc = step_once(h, false, nullptr))) return rc;
+  if ((rc = step_many(h, n - 1))) return rc;
   int64_t rows = 0;
   if ((rc = step_once(h, true, static_cast<double*>(h->partials.p), &rows))) return rc;
   if ((rc = launched(h, reduce_partials(static_cast<double*>(h->partials.p), rows, static_cast<double*>(h->out8.p), h->stream), "stats reduce")))

@@ -51,6 +51,9 @@ struct HostParams {
   unsigned* err;          // device error word of the handle (set by kernels whose bounded waits ran out)
   unsigned inject_extra_tx;                // failure injection: bytes a TMA-fed step waits for beyond its copies
   unsigned long long inject_wait_ns;       // and the limit of its waits then
+  int device;             // the handle's device, its SM count and the bytes of its L2
+  int sms;
+  int64_t l2_bytes;
   cudaStream_t stream;
 };
 
@@ -89,6 +92,9 @@ struct KernelTable {
                       void* dst, double* partials);
   // rows of partial sums that step() with these patterns writes when stats is set
   int64_t (*step_rows)(const HostParams&, int gather, int scatter);
+  // two pull steps from a POST state to a POST state in one pass, where the lattice allows it
+  bool (*step2_ok)(const HostParams&);
+  cudaError_t (*step2)(const HostParams&, const void* src, void* dst);
   cudaError_t (*to_f64)(const HostParams&, int gather, const void* src, double* f);
   cudaError_t (*moments)(const HostParams&, int gather, const void* src, double* rho, double* u);
   cudaError_t (*stats)(const HostParams&, int gather, const void* src, double* partials);
@@ -141,6 +147,7 @@ cudaError_t ade_density(const AdeHost& h, const void* g, double* C);
 // planes of a buffer: dimensions (x, y, z, population), box (box_x, box_rows, 1, 1).
 // Returns false when the driver does not provide the encoder or refuses the layout.
 int device_sm_count();
+int64_t device_l2_bytes();
 // Tuning setting of the TMA-fed step: the environment variable `name` (read once)
 // when set to an integer, else `fallback` (the compiled default).
 int tma_setting(const char* name, int fallback);

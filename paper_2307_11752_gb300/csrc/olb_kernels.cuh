@@ -28,6 +28,7 @@
 #include <cuda_fp16.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <type_traits>
 #include <utility>
 
@@ -248,6 +249,16 @@ struct Store<__nv_bfloat16> {
   __device__ static void st(__nv_bfloat16* p, C v) { *p = __float2bfloat16_rn(v); }
 };
 
+// Constants of the Guo source of the uniform force in the paired FP32 collision
+// (scaled units: F times the storage scale), formed on the host in FP32 in the order
+// of the formulas:
+//   gs[k] = 9 (1 - omega/2) w_k c_k.F,  ga[k] = 3 (1 - omega_odd/2) w_k c_k.F  (k: the
+//   velocities HALF + 1 ..), uf = -3 (1 - omega/2) w for the two moving weights,
+//   src0 = -3 (1 - omega/2) w_0.
+struct PairForce {
+  float force[3], gs[9], ga[9], uf[2], src0;
+};
+
 // Kernel parameters in the compute type C.
 template <class C>
 struct Params {
@@ -278,7 +289,27 @@ struct Params {
   int y0, z0, y1, z1;  // rows covered by the step grid
   int az0, az1;        // active planes: statistics count cells with z in [az0, az1]
   const float* __restrict__ wall_f;  // [256][20]: 6 w_i (c_i . u_w) rounded once to FP32
+  PairForce pf;
 };
+
+template <class L>
+PairForce pair_force(const Params<float>& p, bool trt, float scale) {
+  PairForce r = {};
+  const float gf = 1.0f - 0.5f * p.omega;
+  const float go = trt ? 1.0f - 0.5f * p.omega_minus : gf;
+  for (int a = 0; a < 3; ++a) r.force[a] = p.force[a] * scale;
+  for (int k = 1; k <= L::HALF; ++k) {
+    const float wk = (float)L::w(k);
+    float cF = 0.0f;
+    for (int a = 0; a < L::DIM; ++a)
+      if (L::c(k + L::HALF, a) != 0) cF += (float)L::c(k + L::HALF, a) * r.force[a];
+    r.gs[k - 1] = 9.0f * gf * wk * cF;
+    r.ga[k - 1] = 3.0f * go * wk * cF;
+    r.uf[wk == (float)L::w(1) ? 0 : 1] = -3.0f * gf * wk;
+  }
+  r.src0 = -3.0f * gf * (float)L::w(0);
+  return r;
+}
 
 template <class C>
 Params<C> to_params(const HostParams& h) {
@@ -1236,6 +1267,7 @@ __global__ void __launch_bounds__(256) k_misfit_seed(Params<typename Store<S>::C
 
 #include "olb_pair.cuh"
 #include "olb_tma.cuh"
+#include "olb_march.cuh"
 
 namespace olb {
 
@@ -1250,6 +1282,7 @@ struct Launch {
   static Params<C> params(const HostParams& h) {
     Params<C> p = to_params<C>(h);
     p.all_fluid = h.cls == nullptr ? 1 : 0;
+    if constexpr (!std::is_same<S, double>::value) p.pf = pair_force<L>(p, h.trt, PairStore<S>::SCALE);
     return p;
   }
 
@@ -1438,6 +1471,91 @@ struct Launch {
     return launch_step(k_step<L, S, G, SC, STATS, TRT>, g.dims(), dim3(256), 0, h.stream, params(h),
                        static_cast<const S*>(src), static_cast<S*>(dst), partials);
   }
+  // Tiles of the two-step pass (k_step2) and the planes per block that give the fewest
+  // plane iterations on the SM with most blocks.
+  static int64_t step2_geometry(const HostParams& h, int& xt, int& yt, int& cz) {
+    using M = March<S>;
+    const int nz = h.z1 - h.z0 + 1;
+    xt = (h.nx + M::TX - 1) / M::TX;
+    yt = (h.y1 - h.y0 + M::TY) / M::TY;
+    int64_t cost = INT64_MAX;
+    for (int nc = 1; nc <= nz; ++nc) {
+      const int c = (nz + nc - 1) / nc;
+      const int64_t waves = ((int64_t)xt * yt * ((nz + c - 1) / c) + h.sms - 1) / h.sms;
+      if (waves * (c + 3) < cost) {
+        cost = waves * (c + 3);
+        cz = c;
+      }
+    }
+    return cost;
+  }
+
+  // Whether two pull steps from a POST state run as one pass (k_step2).  It accepts
+  // lattices with a uniform or no force and no link that leaves the domain, nx even,
+  // and pays where single steps are bound by HBM: both buffers together beyond L2.
+  // A plane iteration costs 3.5 to 4.0 us without and 4.8 us with walls on all SMs at
+  // once, the single steps it replaces 6.2 and 6.9 us for the cells of as many full
+  // tiles; so the lattice has to fill its tiles and planes by 0.66 and 0.72.  (128^3
+  // FP32: 47.4 -> 38.3 us a step without walls, cavity 50.5 -> 44.8; 96^3 cavity, in
+  // L2: 24.1 one by one, 27.6 in pairs.)  16-bit storage halves the traffic but not the
+  // instructions: 256^3 without walls 205 -> 198 us, but 28.0 -> 32.5 us at 128^3 (not
+  // much more than L2), and 35.3 -> 38.9 us with walls there; so only without walls and
+  // from four times L2.  The Guo source adds a quarter to the arithmetic
+  // (channel 128^3 50.2 -> 49.0 us, TRT 97.4 -> 96.5 us: not worth the state), so
+  // forced lattices step one by one.
+  static bool step2_ok(const HostParams& h) {
+    if constexpr (std::is_same<S, double>::value || L::DIM != 3) {
+      return false;
+    } else {
+      const bool walls = h.cls != nullptr;
+      if (!pairs_ok(h.nx) || h.ffield != nullptr || h.forced || h.outside_links || h.az0 != 0 || h.az1 != h.nz - 1 ||
+          tma_setting("OLB_TMA", OLB_TMA))
+        return false;
+      if (sizeof(S) == 2 && walls) return false;
+      const uint64_t plane_bytes = (uint64_t)h.pitch * sizeof(S);
+      if (plane_bytes >= (1ull << 32) || (uint64_t)h.nx * h.ny * sizeof(S) >= (1ull << 31)) return false;  // k_step2
+      if (2 * L::Q * plane_bytes <= (sizeof(S) == 2 ? 4 : 1) * (uint64_t)h.l2_bytes) return false;
+      int xt, yt, cz;
+      const int64_t planes = step2_geometry(h, xt, yt, cz);
+      const double cells = (double)h.nx * (h.y1 - h.y0 + 1) * (h.z1 - h.z0 + 1);
+      return cells > (walls ? 0.72 : 0.66) * (double)planes * h.sms * (March<S>::TX * March<S>::TY);
+    }
+  }
+
+  template <bool WALLS, bool TRT>
+  static cudaError_t launch_step2(const HostParams& h, const void* src, void* dst) {
+    using M = March<S>;
+    auto kernel = k_step2<S, WALLS, TRT>;
+    // shared memory above 48 KB is granted once per device
+    static std::atomic<uint64_t> granted{0};
+    const uint64_t bit = uint64_t(1) << (h.device & 63);
+    if (!(granted.load(std::memory_order_relaxed) & bit)) {
+      cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)M::smem());
+      if (e != cudaSuccess) return e;
+      granted.fetch_or(bit, std::memory_order_relaxed);
+    }
+    const Params<float> p = params(h);
+    const MarchBuf<S> pl{static_cast<const S*>(src), static_cast<S*>(dst), (unsigned)(h.pitch * sizeof(S))};
+    int xt, yt, cz;
+    step2_geometry(h, xt, yt, cz);
+    const int nz = h.z1 - h.z0 + 1;
+    return launch_step(kernel, dim3(xt, yt, (nz + cz - 1) / cz), dim3(M::THREADS), M::smem(), h.stream, p, pl,
+                       MarchGeom{cz});
+  }
+
+  // Two pull steps, POST to POST.
+  static cudaError_t step2(const HostParams& h, const void* src, void* dst) {
+    if constexpr (std::is_same<S, double>::value || L::DIM != 3) {
+      return cudaErrorNotSupported;
+    } else {
+      if constexpr (sizeof(S) == 4) {
+        if (h.cls != nullptr)
+          return h.trt ? launch_step2<true, true>(h, src, dst) : launch_step2<true, false>(h, src, dst);
+      }
+      return h.trt ? launch_step2<false, true>(h, src, dst) : launch_step2<false, false>(h, src, dst);
+    }
+  }
+
   template <int G, int SC>
   static cudaError_t step_s(const HostParams& h, bool stats, const void* src, void* dst,
                             double* partials) {
@@ -1540,7 +1658,7 @@ struct Launch {
   }
 
   static const KernelTable* table() {
-    static const KernelTable t = {L::Q,       sizeof(S), sizeof(T), &step,    &step_rows, &to_f64,
+    static const KernelTable t = {L::Q,       sizeof(S), sizeof(T), &step,    &step_rows, &step2_ok, &step2, &to_f64,
                                   &moments,   &stats,    &from_f64, &init_eq, &perturb,
                                   &materialize, &adjoint, &loss_seed, &misfit_seed};
     return &t;

@@ -161,12 +161,6 @@ __device__ __forceinline__ void st_pair(S* plane, const PairNbr& n, int dx, int 
   }
 }
 
-// BGK relaxation with omega w_k folded into the equilibrium's coefficients, per
-// weight class (fewer instructions, a few more live registers).
-#ifndef OLB_FOLD_OMEGA
-#define OLB_FOLD_OMEGA 0
-#endif
-
 // ---------------------------------------------------------------------------------
 // Collision of a pair in scaled units (values are (f - w) * SCALE).
 //   rho_s = SCALE + sum f_s,  u = (j_s + F_s/2) / rho_s,  F_s = SCALE * F,
@@ -174,13 +168,17 @@ __device__ __forceinline__ void st_pair(S* plane, const PairNbr& n, int dx, int 
 // Returns rho_s and u for the wall terms and statistics.
 // ---------------------------------------------------------------------------------
 // TRT = true: the two-relaxation-time operator (see collide in olb_kernels.cuh).
-template <class L, int SCALE_NUM, bool TRT = false>
-__device__ __forceinline__ void collide_pair(const Params<float>& p, F2 gamma, F2 (&f)[L::Q], F2& drho_s,
-                                             F2 (&j_s)[3], F2& rho_s, F2 (&u)[3]) {
+// FORCED: the Guo source with the uniform force; its constants per direction come
+// from the host (PairForce), already as pairs, instead of from ~75 scalar
+// multiplications per pair of cells.
+template <class L, int SCALE_NUM, bool TRT, bool FORCED>
+__device__ __forceinline__ void collide_pair_t(const Params<float>& p, F2 gamma, F2 (&f)[L::Q], F2& drho_s,
+                                               F2 (&j_s)[3], F2& rho_s, F2 (&u)[3]) {
   constexpr float SCALE = (float)SCALE_NUM;
   // moments
   F2 d = f[0];
-  F2 jj[3] = {F2(0.0f), F2(0.0f), F2(0.0f)};
+  F2 jj[3];
+  bool jset[3] = {false, false, false};
 #pragma unroll
   for (int k = 1; k <= L::HALF; ++k) {
     const int kp = k + L::HALF;
@@ -188,10 +186,18 @@ __device__ __forceinline__ void collide_pair(const Params<float>& p, F2 gamma, F
     const F2 a = f[kp] - f[k];
 #pragma unroll
     for (int dd = 0; dd < 3; ++dd) {
-      if (L::c(kp, dd) == 1) jj[dd] = jj[dd] + a;
-      if (L::c(kp, dd) == -1) jj[dd] = jj[dd] - a;
+      if (L::c(kp, dd) == 0) continue;
+      if (!jset[dd]) {
+        jj[dd] = L::c(kp, dd) == 1 ? a : neg(a);
+        jset[dd] = true;
+      } else {
+        jj[dd] = L::c(kp, dd) == 1 ? jj[dd] + a : jj[dd] - a;
+      }
     }
   }
+#pragma unroll
+  for (int dd = 0; dd < 3; ++dd)
+    if (!jset[dd]) jj[dd] = F2(0.0f);
   drho_s = d;
   j_s[0] = jj[0];
   j_s[1] = jj[1];
@@ -202,8 +208,12 @@ __device__ __forceinline__ void collide_pair(const Params<float>& p, F2 gamma, F
   F2 up[3];
 #pragma unroll
   for (int dd = 0; dd < 3; ++dd) {
-    u[dd] = (jj[dd] + F2(p.half_force[dd] * SCALE)) * inv;
-    up[dd] = gamma * u[dd];
+    u[dd] = (FORCED ? jj[dd] + F2(p.half_force[dd] * SCALE) : jj[dd]) * inv;
+    up[dd] = u[dd];
+  }
+  if (p.gamma) {
+#pragma unroll
+    for (int dd = 0; dd < 3; ++dd) up[dd] = gamma * u[dd];
   }
   F2 usq = up[0] * up[0];
   usq = fma2(up[1], up[1], usq);
@@ -215,17 +225,16 @@ __device__ __forceinline__ void collide_pair(const Params<float>& p, F2 gamma, F
   const F2 A = fma2(F2(-1.5f) * rho, usq, d);
   const F2 B = F2(4.5f) * rho;
   const F2 T = F2(3.0f) * rho;
-  const float gf = 1.0f - 0.5f * om;
   F2 uF(0.0f);
-  if (p.forced) {
-    uF = up[0] * F2(p.force[0] * SCALE);
-    uF = fma2(up[1], F2(p.force[1] * SCALE), uF);
-    uF = fma2(up[2], F2(p.force[2] * SCALE), uF);
+  if (FORCED) {
+    uF = up[0] * F2(p.pf.force[0]);
+    uF = fma2(up[1], F2(p.pf.force[1]), uF);
+    uF = fma2(up[2], F2(p.pf.force[2]), uF);
   }
   {
     const float w0 = (float)L::w(0);
     F2 v = fma2(one_m_om, f[0], F2(om * w0) * A);
-    if (p.forced) v = fma2(F2(-3.0f * gf * w0), uF, v);
+    if (FORCED) v = fma2(F2(p.pf.src0), uF, v);
     f[0] = v;
   }
 #pragma unroll
@@ -233,7 +242,6 @@ __device__ __forceinline__ void collide_pair(const Params<float>& p, F2 gamma, F
     const int kp = k + L::HALF;
     const float wk = (float)L::w(k);
     F2 cu(0.0f);
-    float cFs = 0.0f;
     bool first = true;
 #pragma unroll
     for (int dd = 0; dd < L::DIM; ++dd) {
@@ -245,41 +253,42 @@ __device__ __forceinline__ void collide_pair(const Params<float>& p, F2 gamma, F
         } else {
           cu = c > 0 ? cu + up[dd] : cu - up[dd];
         }
-        cFs += c * p.force[dd] * SCALE;
       }
     }
     F2 fp, fm;
-    if (!TRT && OLB_FOLD_OMEGA) {
-      // omega w_k (sym +- anti) with omega w_k folded into A, B and T once per weight
-      // class (the products below are common to the directions of equal weight)
-      const F2 symw = fma2(F2(om * wk * 4.5f) * rho, cu * cu, F2(om * wk) * A);
-      const F2 antiw = F2(om * wk * 3.0f) * rho * cu;
-      fp = fma2(one_m_om, f[kp], symw + antiw);
-      fm = fma2(one_m_om, f[k], symw - antiw);
-    } else if (!TRT) {
+    if (!TRT) {
       const F2 sym = F2(wk) * fma2(B, cu * cu, A);
       const F2 anti = F2(wk) * T * cu;
       fp = fma2(one_m_om, f[kp], omv * (sym + anti));
       fm = fma2(one_m_om, f[k], omv * (sym - anti));
     } else {
-      const F2 sym = F2(wk) * fma2(B, cu * cu, A);
-      const F2 anti = F2(wk) * T * cu;
+      const F2 nsym = F2(-wk) * fma2(B, cu * cu, A);
+      const F2 nanti = F2(-wk) * T * cu;
       // even = omega (f+ - sym), odd = omega_minus (f- - anti), f+- = (f_kp +- f_k)/2
-      const F2 even = omv * fma2(F2(0.5f), f[kp] + f[k], neg(sym));
-      const F2 odd = F2(p.omega_minus) * fma2(F2(0.5f), f[kp] - f[k], neg(anti));
+      const F2 even = omv * fma2(F2(0.5f), f[kp] + f[k], nsym);
+      const F2 odd = F2(p.omega_minus) * fma2(F2(0.5f), f[kp] - f[k], nanti);
       fp = f[kp] - (even + odd);
       fm = f[k] - (even - odd);
     }
-    if (p.forced) {
+    if (FORCED) {
       // Guo: gf w (9 cu cF - 3 u'.F) +- 3 gf w cF   (F in scaled units)
-      const F2 gs = fma2(F2(9.0f * gf * wk * cFs), cu, F2(-3.0f * gf * wk) * uF);
-      const float ga = 3.0f * (TRT ? 1.0f - 0.5f * p.omega_minus : gf) * wk * cFs;
-      fp = fp + gs + F2(ga);
-      fm = fm + gs - F2(ga);
+      const F2 gs = fma2(F2(p.pf.gs[k - 1]), cu, F2(wk == (float)L::w(1) ? p.pf.uf[0] : p.pf.uf[1]) * uF);
+      const F2 ga(p.pf.ga[k - 1]);
+      fp = fp + gs + ga;
+      fm = fm + gs - ga;
     }
     f[kp] = fp;
     f[k] = fm;
   }
+}
+
+template <class L, int SCALE_NUM, bool TRT = false>
+__device__ __forceinline__ void collide_pair(const Params<float>& p, F2 gamma, F2 (&f)[L::Q], F2& drho_s,
+                                             F2 (&j_s)[3], F2& rho_s, F2 (&u)[3]) {
+  if (p.forced)
+    collide_pair_t<L, SCALE_NUM, TRT, true>(p, gamma, f, drho_s, j_s, rho_s, u);
+  else
+    collide_pair_t<L, SCALE_NUM, TRT, false>(p, gamma, f, drho_s, j_s, rho_s, u);
 }
 
 // 6 w_i (c_i . u_w) of wall material m (FP32 table).
