@@ -45,11 +45,6 @@
 #ifndef OLB_STEP_MIN_BLOCKS
 #define OLB_STEP_MIN_BLOCKS 4
 #endif
-// FP64: 2 blocks (<= 128 registers, no spill; at 4 blocks it spills ~390 bytes per
-// thread).  The FP64 step is bound by the FP64 pipe, which 16 warps per SM keep busy.
-#ifndef OLB_STEP64_MIN_BLOCKS
-#define OLB_STEP64_MIN_BLOCKS 2
-#endif
 // Same for the two-cells-per-thread step kernel (FP32 arithmetic), for FP32
 // storage and for 16-bit storage (which needs more cells in flight per byte).
 // FP32: 3 blocks (<= 80 registers) with the bounce-back stores first and their
@@ -259,6 +254,30 @@ struct PairForce {
   float force[3], gs[9], ga[9], uf[2], src0;
 };
 
+// Constants of the FP64 collision (collide_folded), formed once on the host: on this GPU
+// an FP64 instruction of a warp holds an SM's FP64 pipe for 16 cycles, so products of
+// uniform values are not left to the threads.  Weight classes 0: rest, 1, 2: the moving
+// velocities (along an axis, diagonal).
+struct Fold64 {
+  double keep, even, odd;      // 1 - omega, (1 - omega)/2 and (1 - omega_odd)/2
+  double ow[3], b[3], t[3];    // omega w, 4.5 omega w, 3 omega_odd w
+  double gu[3];                // 3 (1 - omega/2) w
+  double gq[9], ga[9];         // 9 (1 - omega/2) w_k c_k.F,  3 (1 - omega_odd/2) w_k c_k.F
+};
+
+// n / d for 0 <= n < 2^31 by one high multiplication (T. Granlund, P. Montgomery,
+// "Division by invariant integers using multiplication", PLDI 1994).
+struct FastDiv {
+  unsigned d, m;
+  int s;
+  FastDiv() = default;
+  explicit FastDiv(unsigned d_) : d(d_), m(0), s(0) {
+    while ((1ull << s) < d) ++s;
+    m = (unsigned)(((1ull << (31 + s)) + d - 1) / d);
+  }
+  __device__ __forceinline__ unsigned div(unsigned n) const { return s == 0 ? n : __umulhi(n, m) >> (s - 1); }
+};
+
 // Kernel parameters in the compute type C.
 template <class C>
 struct Params {
@@ -290,7 +309,40 @@ struct Params {
   int az0, az1;        // active planes: statistics count cells with z in [az0, az1]
   const float* __restrict__ wall_f;  // [256][20]: 6 w_i (c_i . u_w) rounded once to FP32
   PairForce pf;
+  Fold64 fold;      // FP64 only
+  FastDiv by_nx, by_ny;  // FP64 step: flat index over the rows [y0, y1] x [z0, z1]
+  unsigned flat;
 };
+
+template <class L>
+__host__ __device__ constexpr int weight_class(int k) {
+  return k == 0 ? 0 : (L::c(k, 0) * L::c(k, 0) + L::c(k, 1) * L::c(k, 1) + L::c(k, 2) * L::c(k, 2) == 1 ? 1 : 2);
+}
+
+template <class L>
+Fold64 fold64(const Params<double>& p, bool trt) {
+  Fold64 r = {};
+  const double odd = trt ? p.omega_minus : p.omega;
+  const double ge = 1.0 - 0.5 * p.omega, go = 1.0 - 0.5 * odd;
+  r.keep = 1.0 - p.omega;
+  r.even = 0.5 * (1.0 - p.omega);
+  r.odd = 0.5 * (1.0 - odd);
+  for (int k = 0; k < L::Q; ++k) {
+    const int c = weight_class<L>(k);
+    const double w = L::w(k);
+    r.ow[c] = p.omega * w;
+    r.b[c] = 4.5 * p.omega * w;
+    r.t[c] = 3.0 * odd * w;
+    r.gu[c] = 3.0 * ge * w;
+    if (k > L::HALF) {
+      double cF = 0.0;
+      for (int a = 0; a < L::DIM; ++a) cF += L::c(k, a) * p.force[a];
+      r.gq[k - L::HALF - 1] = 9.0 * ge * w * cF;
+      r.ga[k - L::HALF - 1] = 3.0 * go * w * cF;
+    }
+  }
+  return r;
+}
 
 template <class L>
 PairForce pair_force(const Params<float>& p, bool trt, float scale) {
@@ -616,6 +668,87 @@ __device__ __forceinline__ void collide(const Params<C>& p, C gamma, const C (&F
   }
 }
 
+// The FP64 collision with a uniform force: relaxation towards the equilibrium and the
+// source of a pair (k, opp k) by their even and odd halves,
+//   S = omega w (drho - 1.5 rho u'^2) - 3 ge w u'.F + c.u' (4.5 omega w rho c.u' + 9 ge w c.F)
+//   A = 3 omega_odd w rho c.u' + 3 go w c.F      (ge = 1 - omega/2, go = 1 - omega_odd/2)
+//   BGK  f*_k = (1 - omega) f_k + (S + A),  f*_opp = (1 - omega) f_opp + (S - A)
+//   TRT  f*_k, f*_opp = [(1 - omega)/2 (f_k + f_opp) + S] +- [(1 - omega_odd)/2 (f_k - f_opp) + A]
+// About 145 FP64 instructions on D3Q19 with or without force, where collide takes 250
+// with one.  The FP64 pipe bounds the step.
+template <class L, bool TRT>
+__device__ __forceinline__ void collide_folded(const Params<double>& p, double gamma, double (&f)[L::Q], double& drho,
+                                               double (&j)[3], double& rho, double (&u)[3]) {
+  const Fold64& c = p.fold;
+  double s[L::HALF], a[L::HALF];
+  drho = f[0];
+  bool set[3] = {false, false, false};
+  j[0] = j[1] = j[2] = 0.0;
+#pragma unroll
+  for (int k = 0; k < L::HALF; ++k) {
+    const int kp = k + 1 + L::HALF;
+    s[k] = f[k + 1] + f[kp];
+    a[k] = f[kp] - f[k + 1];
+    drho += s[k];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+      if (L::c(kp, d) == 0) continue;
+      if (!set[d])
+        j[d] = L::c(kp, d) == 1 ? a[k] : -a[k];
+      else
+        j[d] = L::c(kp, d) == 1 ? j[d] + a[k] : j[d] - a[k];
+      set[d] = true;
+    }
+  }
+  rho = 1.0 + drho;
+  const double inv = 1.0 / rho;
+  double up[3] = {0.0, 0.0, 0.0};
+#pragma unroll
+  for (int d = 0; d < 3; ++d) u[d] = d < L::DIM ? (j[d] + p.half_force[d]) * inv : 0.0;
+#pragma unroll
+  for (int d = 0; d < L::DIM; ++d) up[d] = u[d];
+  if (p.gamma) {
+#pragma unroll
+    for (int d = 0; d < L::DIM; ++d) up[d] = gamma * u[d];
+  }
+  double usq = up[0] * up[0] + up[1] * up[1];
+  if (L::DIM == 3) usq += up[2] * up[2];
+  const double dr = drho - 1.5 * rho * usq;
+  double base[3] = {c.ow[0] * dr, c.ow[1] * dr, c.ow[2] * dr};
+  if (p.forced) {
+    double uF = up[0] * p.force[0] + up[1] * p.force[1];
+    if (L::DIM == 3) uF += up[2] * p.force[2];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) base[k] -= c.gu[k] * uF;
+  }
+  f[0] = c.keep * f[0] + base[0];
+  const double br[3] = {0.0, c.b[1] * rho, c.b[2] * rho}, tr[3] = {0.0, c.t[1] * rho, c.t[2] * rho};
+#pragma unroll
+  for (int k = 0; k < L::HALF; ++k) {
+    const int kp = k + 1 + L::HALF, w = weight_class<L>(k + 1);
+    double cu = 0.0;
+    bool first = true;
+#pragma unroll
+    for (int d = 0; d < L::DIM; ++d) {
+      if (L::c(kp, d) == 0) continue;
+      if (first)
+        cu = L::c(kp, d) == 1 ? up[d] : -up[d];
+      else
+        cu = L::c(kp, d) == 1 ? cu + up[d] : cu - up[d];
+      first = false;
+    }
+    const double S = cu * (br[w] * cu + c.gq[k]) + base[w], A = tr[w] * cu + c.ga[k];
+    if (TRT) {
+      const double e = c.even * s[k] + S, o = c.odd * a[k] + A;
+      f[kp] = e + o;
+      f[k + 1] = e - o;
+    } else {
+      f[kp] = c.keep * f[kp] + (S + A);
+      f[k + 1] = c.keep * f[k + 1] + (S - A);
+    }
+  }
+}
+
 // ---------------------------------------------------------------------------------
 // Scatter post-collision values f*_i(x) to a buffer with pattern SC.
 //   S_OWN       slot i of x                         -> state POST (next gather G_PULL)
@@ -772,29 +905,57 @@ __device__ __forceinline__ bool on_edge(const Params<C>& p, int x, int y, int z)
 // the cell; it collides and stores.  Links leaving the domain (only when some
 // fluid cell touches a non-periodic domain face) are recognised from the
 // coordinates, again without waiting for a load.
+//
+// FP64: cells are dealt to the threads by a flat index over the rows that hold fluid, so
+// that warps are full at any nx (75 cells a row: 78 % of the lanes in rows of 32), in
+// blocks small enough to reach every SM on small lattices (flat_threads).
+// 75x61x57 channel with force: 152 -> 72 us; 64^2 D2Q9 vortex: 7.9 -> 3.8 us a step.
 template <class L, class S, int G, int SC, bool STATS, bool TRT>
-__global__ void __launch_bounds__(256, std::is_same<S, double>::value ? OLB_STEP64_MIN_BLOCKS : OLB_STEP_MIN_BLOCKS)
+__global__ void __launch_bounds__(std::is_same<S, double>::value ? 128 : 256,
+                                  std::is_same<S, double>::value ? 4 : OLB_STEP_MIN_BLOCKS)
     k_step(Params<typename Store<S>::C> p, const S* src, S* dst, double* partials) {
   using C = typename Store<S>::C;
+  constexpr bool FLAT = std::is_same<S, double>::value;
   C sv[8] = {C(0), C(0), C(0), C(0), C(0), C(0), C(0), C(0)};
   const int tid = threadIdx.x;
   pdl_wait_then_release();
-  const int z = p.z0 + blockIdx.z;
-  const int x = (blockIdx.x << p.tile_shift) + (tid & ((1 << p.tile_shift) - 1));
-  const int y = p.y0 + blockIdx.y * (256 >> p.tile_shift) + (tid >> p.tile_shift);
-  if (x < p.nx && y <= p.y1) {
+  int x, y, z;
+  bool active;
+  if constexpr (FLAT) {
+    const unsigned id = blockIdx.x * blockDim.x + tid;
+    const unsigned r = p.by_nx.div(id), zz = p.by_ny.div(r);
+    x = (int)(id - r * p.by_nx.d);
+    y = p.y0 + (int)(r - zz * p.by_ny.d);
+    z = p.z0 + (int)zz;
+    active = id < p.flat;
+  } else {
+    z = p.z0 + blockIdx.z;
+    x = (blockIdx.x << p.tile_shift) + (tid & ((1 << p.tile_shift) - 1));
+    y = p.y0 + blockIdx.y * (256 >> p.tile_shift) + (tid >> p.tile_shift);
+    active = x < p.nx && y <= p.y1;
+  }
+  if (active) {
     const Nbr n = make_nbr<L>(p, x, y, z);
     const uint32_t w = p.all_fluid ? kWordFluid : p.word[n.cell];
     C f[L::Q];
     gather_bulk<L, S, G>(p, src, n, f);
     const C gamma = p.gamma ? p.gamma[n.cell] : C(1);
-    C F[3];
-    force_at(p, n.cell, F);
     const bool edge = p.outside_links && on_edge<L>(p, x, y, z);
     if (edge) gather_outside<L, S, G>(p, src, n, f);
     C drho, j[3], rho, u[3];
-    moments<L>(f, drho, j);
-    collide<L, C, TRT>(p, gamma, F, f, drho, j, rho, u);
+    bool done = false;
+    if constexpr (FLAT) {
+      if (!p.ffield) {
+        collide_folded<L, TRT>(p, gamma, f, drho, j, rho, u);
+        done = true;
+      }
+    }
+    if (!done) {
+      C F[3];
+      force_at(p, n.cell, F);
+      moments<L>(f, drho, j);
+      collide<L, C, TRT>(p, gamma, F, f, drho, j, rho, u);
+    }
     if (w & kWordFluid) {
       const uint32_t pm = w & (kWordLinks | kWordMoving);
       const int cls = edge ? 3 : (pm ? 2 : 1);
@@ -912,6 +1073,31 @@ __global__ void __launch_bounds__(256) k_init_eq(Params<typename Store<S>::C> p,
     for (int d = 0; d < L::DIM; ++d) u[d] = (C)u_in[d * N + cell];
   }
   const C usq = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
+  if constexpr (sizeof(C) == sizeof(double)) {
+    // even and odd halves of each pair: half the FP64 instructions (the bound) of the
+    // formula below
+    Store<S>::st(dst + cell, (C)L::w(0) * (drho - C(1.5) * rho * usq));
+    const C r45 = C(4.5) * rho, r3 = C(3) * rho, e0 = drho - C(1.5) * rho * usq;
+#pragma unroll
+    for (int k = 1; k <= L::HALF; ++k) {
+      const int kp = k + L::HALF;
+      C cu = C(0);
+      bool first = true;
+#pragma unroll
+      for (int d = 0; d < L::DIM; ++d) {
+        if (L::c(kp, d) == 0) continue;
+        if (first)
+          cu = L::c(kp, d) == 1 ? u[d] : -u[d];
+        else
+          cu = L::c(kp, d) == 1 ? cu + u[d] : cu - u[d];
+        first = false;
+      }
+      const C e = r45 * cu * cu + e0, o = r3 * cu;
+      Store<S>::st(dst + kp * (size_t)p.pitch + cell, (C)L::w(k) * (e + o));
+      Store<S>::st(dst + k * (size_t)p.pitch + cell, (C)L::w(k) * (e - o));
+    }
+    return;
+  }
 #pragma unroll
   for (int i = 0; i < L::Q; ++i) {
     const C cu = L::c(i, 0) * u[0] + L::c(i, 1) * u[1] + L::c(i, 2) * u[2];
@@ -1282,7 +1468,14 @@ struct Launch {
   static Params<C> params(const HostParams& h) {
     Params<C> p = to_params<C>(h);
     p.all_fluid = h.cls == nullptr ? 1 : 0;
-    if constexpr (!std::is_same<S, double>::value) p.pf = pair_force<L>(p, h.trt, PairStore<S>::SCALE);
+    if constexpr (!std::is_same<S, double>::value) {
+      p.pf = pair_force<L>(p, h.trt, PairStore<S>::SCALE);
+    } else {
+      p.fold = fold64<L>(p, h.trt);
+      p.by_nx = FastDiv(h.nx);
+      p.by_ny = FastDiv(h.y1 - h.y0 + 1);
+      p.flat = (unsigned)((int64_t)h.nx * (h.y1 - h.y0 + 1) * (h.z1 - h.z0 + 1));
+    }
     return p;
   }
 
@@ -1424,7 +1617,20 @@ struct Launch {
       const int b = h.trt ? tma_blocks_for<true, true>(h, tg) : tma_blocks_for<true, false>(h, tg);
       if (b >= 1) return b;
     }
-    return make_step_grid(h, !std::is_same<S, double>::value && pairs_ok(h.nx) && h.ffield == nullptr).blocks();
+    if constexpr (std::is_same<S, double>::value) return flat_blocks(h);
+    return make_step_grid(h, pairs_ok(h.nx) && h.ffield == nullptr).blocks();
+  }
+
+  // FP64 step: threads per block, so that a small lattice still has a block for most
+  // SMs (the FP64 pipe is the bound: idle SMs are lost), and blocks.
+  static int flat_threads(const HostParams& h) {
+    const int64_t cells = (int64_t)h.nx * (h.y1 - h.y0 + 1) * (h.z1 - h.z0 + 1);
+    return cells >= 128 * 8 * (int64_t)h.sms ? 128 : (cells >= 64 * 4 * (int64_t)h.sms ? 64 : 32);
+  }
+  static int64_t flat_blocks(const HostParams& h) {
+    const int64_t cells = (int64_t)h.nx * (h.y1 - h.y0 + 1) * (h.z1 - h.z0 + 1);
+    const int t = flat_threads(h);
+    return (cells + t - 1) / t;
   }
 
   template <int G, int SC, bool STATS, bool TRT>
@@ -1467,6 +1673,9 @@ struct Launch {
                            partials);
       }
     }
+    if constexpr (std::is_same<S, double>::value)
+      return launch_step(k_step<L, S, G, SC, STATS, TRT>, dim3((unsigned)flat_blocks(h)), dim3(flat_threads(h)), 0,
+                         h.stream, params(h), static_cast<const S*>(src), static_cast<S*>(dst), partials);
     const StepGrid g = make_step_grid(h, false);
     return launch_step(k_step<L, S, G, SC, STATS, TRT>, g.dims(), dim3(256), 0, h.stream, params(h),
                        static_cast<const S*>(src), static_cast<S*>(dst), partials);
