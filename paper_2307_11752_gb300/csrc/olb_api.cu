@@ -1445,6 +1445,7 @@ struct olb_ade {
   double tau = 1.0;
   double vu[3] = {0.0, 0.0, 0.0};
   bool has_vfield = false;
+  bool vfield_t = false;   // the field is in the storage type (it came from a fluid lattice)
   bool has_bc = false;     // olb_ade_set_material was called
   unsigned periodic = 7u;
   size_t elem() const { return dtype == OLB_F64 ? sizeof(double) : sizeof(float); }
@@ -1459,7 +1460,8 @@ struct olb_ade {
     a.ncell = ncell;
     a.omega = 1.0 / tau;
     for (int k = 0; k < 3; ++k) a.vu[k] = vu[k];
-    a.vf = has_vfield ? static_cast<const double*>(vfield.p) : nullptr;
+    a.vf = has_vfield && !vfield_t ? static_cast<const double*>(vfield.p) : nullptr;
+    a.vt = has_vfield && vfield_t ? vfield.p : nullptr;
     a.mat = has_bc ? static_cast<const uint8_t*>(mat.p) : nullptr;
     a.lmask = has_bc ? static_cast<const uint8_t*>(lmask.p) : nullptr;
     a.wall_C = has_bc ? static_cast<const double*>(wallC.p) : nullptr;
@@ -1566,6 +1568,7 @@ int olb_ade_set_velocity(olb_ade_handle h, const double v[3], const double* v_fi
     OLB_CUDA(cudaMemcpyAsync(h->vfield.p, v_field, bytes, cudaMemcpyDefault, h->stream), "velocity copy");
     OLB_CUDA(cudaStreamSynchronize(h->stream), "velocity sync");
     h->has_vfield = true;
+    h->vfield_t = false;
   } else {
     for (int a = 0; a < 3; ++a) h->vu[a] = (h->q == 5 && a == 2) ? 0.0 : v[a];
     h->has_vfield = false;
@@ -1632,7 +1635,7 @@ int olb_ade_set_velocity_from(olb_ade_handle h, olb_handle fluid) {
   if ((rc = check(fluid))) return rc;
   if (fluid->nx != h->nx || fluid->ny != h->ny || fluid->nz != h->nz || fluid->dim != (h->q == 5 ? 2 : 3))
     return fail(OLB_ERR_ARG, "the fluid lattice does not match the advection-diffusion lattice");
-  const size_t bytes = 3 * (size_t)h->ncell * sizeof(double);
+  const size_t bytes = 3 * (size_t)h->ncell * h->elem();
   if ((rc = h->vfield.reserve(bytes))) return rc;
   // the fluid's state is final on its own stream; the moments run on this handle's
   cudaEvent_t ev;
@@ -1643,10 +1646,10 @@ int olb_ade_set_velocity_from(olb_ade_handle h, olb_handle fluid) {
   OLB_CUDA(e, "stream order");
   HostParams p = fluid->params();
   p.stream = h->stream;
-  OLB_CUDA(fluid->kt->moments(p, gather_of(fluid->repr), fluid->buf[fluid->cur].p, nullptr,
-                              static_cast<double*>(h->vfield.p)),
+  OLB_CUDA(fluid->kt->velocity(p, gather_of(fluid->repr), fluid->buf[fluid->cur].p, h->vfield.p, h->dtype == OLB_F64),
            "fluid velocity");
   h->has_vfield = true;
+  h->vfield_t = true;
   return OLB_OK;
 }
 

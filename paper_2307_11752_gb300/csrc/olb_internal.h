@@ -82,6 +82,19 @@ inline bool pairs_ok(int) { return false; }
 inline bool pairs_ok(int nx) { return nx % 2 == 0; }
 #endif
 
+// n / d for 0 <= n < 2^31 by one high multiplication (T. Granlund, P. Montgomery,
+// "Division by invariant integers using multiplication", PLDI 1994).
+struct FastDiv {
+  unsigned d, m;
+  int s;
+  FastDiv() = default;
+  explicit FastDiv(unsigned d_) : d(d_), m(0), s(0) {
+    while ((1ull << s) < d) ++s;
+    m = (unsigned)(((1ull << (31 + s)) + d - 1) / d);
+  }
+  __device__ __forceinline__ unsigned div(unsigned n) const { return s == 0 ? n : __umulhi(n, m) >> (s - 1); }
+};
+
 // Launchers of one (lattice, storage type) pair.  Each returns the CUDA error of
 // the launch.  `partials` receives one row of 8 doubles per block (reductions).
 struct KernelTable {
@@ -97,6 +110,8 @@ struct KernelTable {
   cudaError_t (*step2)(const HostParams&, const void* src, void* dst);
   cudaError_t (*to_f64)(const HostParams&, int gather, const void* src, double* f);
   cudaError_t (*moments)(const HostParams&, int gather, const void* src, double* rho, double* u);
+  // the velocity alone, [3][cells] in double or float
+  cudaError_t (*velocity)(const HostParams&, int gather, const void* src, void* u, bool f64);
   cudaError_t (*stats)(const HostParams&, int gather, const void* src, double* partials);
   cudaError_t (*from_f64)(const HostParams&, const double* f, void* dst);
   cudaError_t (*init_eq)(const HostParams&, const double* rho, const double* u, void* dst);
@@ -131,6 +146,7 @@ struct AdeHost {
   double omega;
   double vu[3];           // uniform advection velocity (used when vf is null)
   const double* vf;       // per-cell velocity [3][ncell] or nullptr
+  const void* vt;         // the same in the storage type, or nullptr (takes precedence)
   // boundaries (all null: every cell bulk, every axis periodic)
   const uint8_t* mat;     // per cell: 1 bulk, 0 no-flux wall, 2..255 Dirichlet cell
   const uint8_t* lmask;   // per cell: bit i when link i of a bulk cell hits a non-bulk cell or leaves the domain

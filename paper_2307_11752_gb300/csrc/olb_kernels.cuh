@@ -265,19 +265,6 @@ struct Fold64 {
   double gq[9], ga[9];         // 9 (1 - omega/2) w_k c_k.F,  3 (1 - omega_odd/2) w_k c_k.F
 };
 
-// n / d for 0 <= n < 2^31 by one high multiplication (T. Granlund, P. Montgomery,
-// "Division by invariant integers using multiplication", PLDI 1994).
-struct FastDiv {
-  unsigned d, m;
-  int s;
-  FastDiv() = default;
-  explicit FastDiv(unsigned d_) : d(d_), m(0), s(0) {
-    while ((1ull << s) < d) ++s;
-    m = (unsigned)(((1ull << (31 + s)) + d - 1) / d);
-  }
-  __device__ __forceinline__ unsigned div(unsigned n) const { return s == 0 ? n : __umulhi(n, m) >> (s - 1); }
-};
-
 // Kernel parameters in the compute type C.
 template <class C>
 struct Params {
@@ -966,6 +953,33 @@ __global__ void __launch_bounds__(std::is_same<S, double>::value ? 128 : 256,
     }
   }
   if (STATS) block_reduce_row(sv, partials + 8 * block_linear(), false);
+}
+
+// Velocity u = (j + F/2)/rho of the current state in the type V (the advection field of
+// a scalar lattice): k_moments' values without the density and, for FP32, without 24
+// bytes of FP64 per cell written here and read back by every scalar step.
+template <class L, class S, int G, class V>
+__global__ void __launch_bounds__(256) k_velocity(Params<typename Store<S>::C> p, const S* src, V* u_out) {
+  using C = typename Store<S>::C;
+  const int x = blockIdx.x * blockDim.x + threadIdx.x;
+  const int y = blockIdx.y * blockDim.y + threadIdx.y;
+  if (x >= p.nx || y >= p.ny) return;
+  const Nbr n = make_nbr<L>(p, x, y, blockIdx.z);
+  const int cls = p.all_fluid ? 1 : p.cls[n.cell];
+  const size_t N = (size_t)p.ncell;
+  C u[3] = {C(0), C(0), C(0)};
+  if (cls != 0) {
+    C f[L::Q];
+    gather<L, S, G>(p, src, n, cls, f);
+    C drho, j[3], F[3];
+    moments<L>(f, drho, j);
+    force_at(p, n.cell, F);
+    const C rho = C(1) + drho;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) u[d] = (j[d] + C(0.5) * F[d]) / rho;
+  }
+#pragma unroll
+  for (int d = 0; d < 3; ++d) u_out[d * N + n.cell] = (V)u[d];
 }
 
 // Canonical f(t) = f_shifted + w in double ([q][cells]); non-fluid cells 0.
@@ -1810,6 +1824,21 @@ struct Launch {
                              double* u) {
     OLB_BY_GATHER(k_moments, static_cast<const S*>(src), rho, u);
   }
+  static cudaError_t velocity(const HostParams& h, int gather, const void* src, void* u, bool f64) {
+    Grid g = make_grid(h.nx, h.ny, h.nz);
+    auto run = [&](auto* out) {
+      using V = std::remove_pointer_t<decltype(out)>;
+      const S* s = static_cast<const S*>(src);
+      if (gather == G_OWN)
+        k_velocity<L, S, G_OWN><<<g.grid, g.block, 0, h.stream>>>(params(h), s, static_cast<V*>(u));
+      else if (gather == G_PULL)
+        k_velocity<L, S, G_PULL><<<g.grid, g.block, 0, h.stream>>>(params(h), s, static_cast<V*>(u));
+      else
+        k_velocity<L, S, G_PULL_SWAP><<<g.grid, g.block, 0, h.stream>>>(params(h), s, static_cast<V*>(u));
+      return cudaGetLastError();
+    };
+    return f64 ? run(static_cast<double*>(nullptr)) : run(static_cast<float*>(nullptr));
+  }
   static cudaError_t stats(const HostParams& h, int gather, const void* src, double* partials) {
     OLB_BY_GATHER(k_stats, static_cast<const S*>(src), partials);
   }
@@ -1868,7 +1897,7 @@ struct Launch {
 
   static const KernelTable* table() {
     static const KernelTable t = {L::Q,       sizeof(S), sizeof(T), &step,    &step_rows, &step2_ok, &step2, &to_f64,
-                                  &moments,   &stats,    &from_f64, &init_eq, &perturb,
+                                  &moments,   &velocity,  &stats,    &from_f64, &init_eq, &perturb,
                                   &materialize, &adjoint, &loss_seed, &misfit_seed};
     return &t;
   }
