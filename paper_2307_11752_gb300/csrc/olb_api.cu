@@ -706,11 +706,41 @@ int adjoint_sweep(olb_handle h, int64_t n_steps, int64_t K, Seed&& seed, double 
   // forward sweep with checkpoints (pull pattern)
   const int saved_scheme = h->scheme;
   h->scheme = OLB_PULL;
+  // The last segment steps through the segment's slots, so that the reverse sweep finds
+  // its states there: of n steps, n - K and not n are computed twice.
+  std::vector<const void*> slot(K);
+  std::vector<int> srepr(K);
+  auto through_slots = [&](int64_t s, int64_t ks) {
+    slot[0] = ckpt[s].p;
+    srepr[0] = ckpt_repr[s];
+    for (int64_t k = 1; k < ks; ++k) {
+      const int g = srepr[k - 1] == PRE ? G_OWN : G_PULL;
+      if (int e = launched(h, h->kt->step(h->params(), g, S_OWN, false, slot[k - 1], seg[k].p, nullptr), "recompute"))
+        return e;
+      slot[k] = seg[k].p;
+      srepr[k] = POST;
+    }
+    return (int)OLB_OK;
+  };
+  auto last_segment = [&](int64_t ks) {
+    if (int e = through_slots(nseg - 1, ks)) return e;
+    const int g = srepr[ks - 1] == PRE ? G_OWN : G_PULL;
+    if (int e = launched(h, h->kt->step(h->params(), g, S_OWN, false, slot[ks - 1], h->buf[h->cur].p, nullptr), "step"))
+      return e;
+    h->repr = POST;
+    h->time += ks;
+    return (int)OLB_OK;
+  };
   for (int64_t s = 0; s < nseg; ++s) {
     OLB_CUDA(cudaMemcpyAsync(ckpt[s].p, h->buf[h->cur].p, sb, cudaMemcpyDeviceToDevice, h->stream), "checkpoint");
     ckpt_repr[s] = h->repr;
     const int64_t ks = std::min<int64_t>(K, n_steps - s * K);
-    if ((rc = step_many(h, ks))) {
+    if (s + 1 < nseg) {
+      rc = step_many(h, ks);
+    } else {
+      rc = last_segment(ks);
+    }
+    if (rc) {
       h->scheme = saved_scheme;
       return rc;
     }
@@ -733,16 +763,7 @@ int adjoint_sweep(olb_handle h, int64_t n_steps, int64_t K, Seed&& seed, double 
   int li = 0;
   for (int64_t s = nseg - 1; s >= 0; --s) {
     const int64_t ks = std::min<int64_t>(K, n_steps - s * K);
-    std::vector<const void*> slot(ks);
-    std::vector<int> srepr(ks);
-    slot[0] = ckpt[s].p;
-    srepr[0] = ckpt_repr[s];
-    for (int64_t k = 1; k < ks; ++k) {
-      const int g = srepr[k - 1] == PRE ? G_OWN : G_PULL;
-      if ((rc = launched(h, kt->step(p, g, S_OWN, false, slot[k - 1], seg[k].p, nullptr), "recompute"))) return rc;
-      slot[k] = seg[k].p;
-      srepr[k] = POST;
-    }
+    if (s + 1 < nseg && (rc = through_slots(s, ks))) return rc;
     for (int64_t k = ks - 1; k >= 0; --k) {
       const int g = srepr[k] == PRE ? G_OWN : G_PULL;
       if ((rc = launched(h, kt->adjoint(p, g, slot[k], lam[li].p, lam[1 - li].p, static_cast<double*>(dg.p),
@@ -1354,14 +1375,12 @@ int adjoint_plane(olb_handle h, int64_t n_steps, int64_t K, const olb_objective*
   const int ext[3] = {h->nx, h->ny, h->nz};
   if (obj->plane_index < 0 || obj->plane_index >= ext[obj->plane_axis])
     return fail(OLB_ERR_ARG, "objective plane index out of range");
-  int64_t count = 0;
-  for (int z = 0; z < h->nz; ++z)
-    for (int y = 0; y < h->ny; ++y)
-      for (int x = 0; x < h->nx; ++x) {
-        const int c[3] = {x, y, z};
-        if (c[obj->plane_axis] == obj->plane_index && h->h_mat[((int64_t)z * h->ny + y) * h->nx + x] == OLB_MAT_FLUID)
-          ++count;
-      }
+  int64_t count = 0;  // fluid cells of the plane
+  const int pa = obj->plane_axis, pi = obj->plane_index;
+  for (int z = pa == 2 ? pi : 0; z < (pa == 2 ? pi + 1 : h->nz); ++z)
+    for (int y = pa == 1 ? pi : 0; y < (pa == 1 ? pi + 1 : h->ny); ++y)
+      for (int x = pa == 0 ? pi : 0; x < (pa == 0 ? pi + 1 : h->nx); ++x)
+        count += h->h_mat[((int64_t)z * h->ny + y) * h->nx + x] == OLB_MAT_FLUID;
   if (count == 0) return fail(OLB_ERR_ARG, "objective plane holds no fluid cell");
   const double inv_count = 1.0 / (double)count;
   auto seed = [&](const HostParams& p, const void* state, void* lam0, double* dforce, double* partials) {

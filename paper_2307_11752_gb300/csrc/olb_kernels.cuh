@@ -807,7 +807,7 @@ __device__ __forceinline__ void scatter(const Params<typename Store<S>::C>& p, S
 // type, block and global stages in double.
 // ---------------------------------------------------------------------------------
 template <class C>
-__device__ __forceinline__ void block_reduce_row(C (&v)[8], double* row, bool accumulate) {
+__device__ __forceinline__ void block_reduce_row(C (&v)[8], double* row) {
   __shared__ double sh[32][8];
   const int tid = threadIdx.x + blockDim.x * threadIdx.y;
   const int lane = tid & 31, warp = tid >> 5;
@@ -828,11 +828,25 @@ __device__ __forceinline__ void block_reduce_row(C (&v)[8], double* row, bool ac
   if (tid < 8) {
     double acc = sh[0][tid];
     for (int w = 1; w < nwarps; ++w) acc = (tid == 5) ? fmax(acc, sh[w][tid]) : acc + sh[w][tid];
-    if (accumulate) {
-      row[tid] = (tid == 5) ? fmax(row[tid], acc) : row[tid] + acc;
-    } else {
-      row[tid] = acc;
-    }
+    row[tid] = acc;
+  }
+}
+
+// The same for one sum per thread, added to entry 0 of the row (the adjoint's dL/domega:
+// the other seven entries would take as many shuffles as a tenth of its instructions).
+template <class C>
+__device__ __forceinline__ void block_add_one(C v, double* row) {
+  __shared__ double sh[32];
+  const int tid = threadIdx.x + blockDim.x * threadIdx.y;
+  const int nwarps = (blockDim.x * blockDim.y + 31) >> 5;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if ((tid & 31) == 0) sh[tid >> 5] = (double)v;
+  __syncthreads();
+  if (tid == 0) {
+    double acc = sh[0];
+    for (int w = 1; w < nwarps; ++w) acc += sh[w];
+    row[0] += acc;
   }
 }
 
@@ -952,7 +966,7 @@ __global__ void __launch_bounds__(std::is_same<S, double>::value ? 128 : 256,
       solid_fill<L, S, SC>(p, dst, n, w & kWordLinks);
     }
   }
-  if (STATS) block_reduce_row(sv, partials + 8 * block_linear(), false);
+  if (STATS) block_reduce_row(sv, partials + 8 * block_linear());
 }
 
 // Velocity u = (j + F/2)/rho of the current state in the type V (the advection field of
@@ -1054,7 +1068,7 @@ __global__ void __launch_bounds__(256) k_stats(Params<typename Store<S>::C> p, c
       stats_of(drho, j, u, sv);
     }
   }
-  block_reduce_row(sv, partials + 8 * block_linear(), false);
+  block_reduce_row(sv, partials + 8 * block_linear());
 }
 
 // Stored (shifted) populations from canonical double populations, own slots.
@@ -1194,7 +1208,7 @@ __global__ void __launch_bounds__(256) k_adjoint(Params<typename Store<S>::C> p,
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y * blockDim.y + threadIdx.y;
   const size_t N = (size_t)p.pitch;
-  C sv[8] = {C(0), C(0), C(0), C(0), C(0), C(0), C(0), C(0)};
+  C dom = C(0);  // dL/domega
   pdl_wait_then_release();  // launched like the step kernels (the sweep alternates them)
   if (x < p.nx && y < p.ny) {
     const Nbr n = make_nbr<L>(p, x, y, blockIdx.z);
@@ -1340,14 +1354,14 @@ __global__ void __launch_bounds__(256) k_adjoint(Params<typename Store<S>::C> p,
           lf_odd += C(0.5) * (ls[k] - ls[k + L::HALF]) * (f[k] - f[k + L::HALF]);
         const C src_w = C(3) * dwm * m1F - C(3) * m0 * uF + C(9) * uM2F;
         const C Aex_w = C(3) * dwm * m1u + C(4.5) * um2u - C(1.5) * m0 * usq;
-        sv[0] = m0 * drho + rho * Aex_w - (lf - lf_odd) - dwm * lf_odd - C(0.5) * src_w;
+        dom = m0 * drho + rho * Aex_w - (lf - lf_odd) - dwm * lf_odd - C(0.5) * src_w;
       } else {
         const C src_moment = C(3) * m1F - C(3) * m0 * uF + C(9) * uM2F;
-        sv[0] = m0 * drho + rho * Aex - lf - C(0.5) * src_moment;
+        dom = m0 * drho + rho * Aex - lf - C(0.5) * src_moment;
       }
     }
   }
-  block_reduce_row(sv, partials + 8 * block_linear(), true);
+  block_add_one(dom, partials + 8 * block_linear());
 }
 
 // Objective (mean u[comp] over fluid cells of a plane) and its gradient seed
@@ -1400,7 +1414,7 @@ __global__ void __launch_bounds__(256) k_loss_seed(Params<typename Store<S>::C> 
       }
     }
   }
-  block_reduce_row(sv, partials + 8 * block_linear(), false);
+  block_reduce_row(sv, partials + 8 * block_linear());
 }
 
 // Seed of the adjoint for the velocity misfit J = 1/2 sum over the fluid cells of
@@ -1460,7 +1474,7 @@ __global__ void __launch_bounds__(256) k_misfit_seed(Params<typename Store<S>::C
       }
     }
   }
-  block_reduce_row(sv, partials + 8 * block_linear(), false);
+  block_reduce_row(sv, partials + 8 * block_linear());
 }
 
 }  // namespace olb

@@ -675,7 +675,7 @@ __global__ void __launch_bounds__(256, TRT ? PairStore<S>::MIN_BLOCKS_TRT
     if (p.gamma) gamma = F2(*reinterpret_cast<const float2*>(p.gamma + cell));
     pair_update<L, S, G, SC, STATS, WALLS, TRT>(p, pl, n, x0, y, z, w, gamma, f, sv);
   }
-  if (STATS) block_reduce_row(sv, partials + 8 * block_linear(), false);
+  if (STATS) block_reduce_row(sv, partials + 8 * block_linear());
 }
 
 }  // namespace olb

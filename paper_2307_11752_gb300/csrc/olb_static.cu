@@ -70,7 +70,7 @@ __global__ void __launch_bounds__(256) k_stats_canonical(const double* __restric
     const double u[3] = {(j[0] + hfx) / rho, (j[1] + hfy) / rho, (j[2] + hfz) / rho};
     olb::stats_of(drho, j, u, sv);
   }
-  olb::block_reduce_row(sv, rows + 8 * (int64_t)blockIdx.x, false);
+  olb::block_reduce_row(sv, rows + 8 * (int64_t)blockIdx.x);
 }
 
 // Sum the rows in a fixed order and write the 7 statistics of olb_diagnostics.

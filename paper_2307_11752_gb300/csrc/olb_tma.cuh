@@ -310,7 +310,7 @@ __global__ void __launch_bounds__(256, 2)
     }
   }
   if (!g.release_early) pdl_release();
-  if (STATS) block_reduce_row(sv, partials + 8 * (int64_t)blockIdx.x, false);
+  if (STATS) block_reduce_row(sv, partials + 8 * (int64_t)blockIdx.x);
 }
 
 }  // namespace olb
