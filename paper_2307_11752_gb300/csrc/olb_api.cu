@@ -591,19 +591,23 @@ int step_once(olb_handle h, bool stats, double* partials, int64_t* rows = nullpt
   return OLB_OK;
 }
 
-// n steps in the handle's scheme without statistics: pairs of pull steps in one pass
+// n steps in the handle's scheme without statistics: several pull steps per launch
 // where the lattice allows it, else step by step.
 int step_many(olb_handle h, int64_t n) {
   int rc;
   while (n > 0) {
     if (n >= 2 && h->scheme == OLB_PULL && h->repr == POST && !h->inject_tx) {
       const HostParams p = h->params();
-      if (h->kt->step2_ok(p)) {
+      const int strip = h->kt->strip_steps(p);
+      const int k = strip ? (int)std::min<int64_t>(strip, n) : (h->kt->step2_ok(p) ? 2 : 0);
+      if (k) {
         if ((rc = ensure_other(h))) return rc;
-        if ((rc = launched(h, h->kt->step2(p, h->buf[h->cur].p, h->buf[1 - h->cur].p), "step pair"))) return rc;
+        const void* a = h->buf[h->cur].p;
+        void* b = h->buf[1 - h->cur].p;
+        if ((rc = launched(h, strip ? h->kt->strip(p, k, a, b) : h->kt->step2(p, a, b), "steps"))) return rc;
         h->cur = 1 - h->cur;
-        h->time += 2;
-        n -= 2;
+        h->time += k;
+        n -= k;
         continue;
       }
     }

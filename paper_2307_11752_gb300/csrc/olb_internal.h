@@ -108,6 +108,9 @@ struct KernelTable {
   // two pull steps from a POST state to a POST state in one pass, where the lattice allows it
   bool (*step2_ok)(const HostParams&);
   cudaError_t (*step2)(const HostParams&, const void* src, void* dst);
+  // n <= strip_steps() pull steps (0: not offered) from a POST state to a POST state in one launch
+  int (*strip_steps)(const HostParams&);
+  cudaError_t (*strip)(const HostParams&, int n, const void* src, void* dst);
   cudaError_t (*to_f64)(const HostParams&, int gather, const void* src, double* f);
   cudaError_t (*moments)(const HostParams&, int gather, const void* src, double* rho, double* u);
   // the velocity alone, [3][cells] in double or float

@@ -1482,6 +1482,7 @@ __global__ void __launch_bounds__(256) k_misfit_seed(Params<typename Store<S>::C
 #include "olb_pair.cuh"
 #include "olb_tma.cuh"
 #include "olb_march.cuh"
+#include "olb_strip.cuh"
 
 namespace olb {
 
@@ -1780,6 +1781,39 @@ struct Launch {
                        MarchGeom{cz});
   }
 
+  // Steps that one launch of k_strip takes (0: the lattice has no such path).  Halo 8
+  // while its 48 x 16 parts fill the SMs at most twice over (launches count: 256^2 FP32
+  // 2.32 -> 1.62 us a step, FP16 2.19 -> 1.62), else halo 4, parts of 56 x 24 (700 x 500
+  // FP32 4.46 -> 2.94, 1024^2 8.62 -> 7.84, 2048^2 45.9 -> 28.9).  With less traffic (16-bit
+  // storage) or more arithmetic (TRT) the large lattice has to be beyond L2: 2048^2
+  // FP16 36.0 -> 27.4 us, but 1024^2 FP16 7.54 -> 7.82, FP32 TRT 8.71 -> 8.75.
+  static int strip_steps(const HostParams& h) {
+    if constexpr (std::is_same<S, double>::value || L::DIM != 2) {
+      return 0;
+    } else {
+      if (h.cls != nullptr || !pairs_ok(h.nx) || h.ffield != nullptr || h.az0 != 0 || h.az1 != h.nz - 1 ||
+          tma_setting("OLB_TMA", OLB_TMA))
+        return 0;
+      const int64_t parts = (int64_t)((h.nx + 47) / 48) * ((h.ny + 15) / 16);
+      if (parts <= 2 * (int64_t)h.sms) return 8;
+      if ((sizeof(S) == 2 || h.trt) && (int64_t)(2 * L::Q * sizeof(S)) * h.pitch <= h.l2_bytes) return 0;
+      return 4;
+    }
+  }
+
+  // n <= strip_steps(h) pull steps, POST to POST.
+  static cudaError_t strip(const HostParams& h, int n, const void* src, void* dst) {
+    if constexpr (std::is_same<S, double>::value || L::DIM != 2) {
+      return cudaErrorNotSupported;
+    } else {
+      const StripGeom g{strip_steps(h), n};
+      const int ow = kStripX - 2 * g.halo, oh = kStripY - 2 * g.halo;
+      const dim3 grid((h.nx + ow - 1) / ow, (h.ny + oh - 1) / oh), block(32 * kStripWarps);
+      return launch_step(h.trt ? k_strip<S, true> : k_strip<S, false>, grid, block, 0, h.stream, params(h),
+                         static_cast<const S*>(src), static_cast<S*>(dst), g);
+    }
+  }
+
   // Two pull steps, POST to POST.
   static cudaError_t step2(const HostParams& h, const void* src, void* dst) {
     if constexpr (std::is_same<S, double>::value || L::DIM != 3) {
@@ -1910,7 +1944,7 @@ struct Launch {
   }
 
   static const KernelTable* table() {
-    static const KernelTable t = {L::Q,       sizeof(S), sizeof(T), &step,    &step_rows, &step2_ok, &step2, &to_f64,
+    static const KernelTable t = {L::Q,       sizeof(S), sizeof(T), &step,    &step_rows, &step2_ok, &step2, &strip_steps, &strip, &to_f64,
                                   &moments,   &velocity,  &stats,    &from_f64, &init_eq, &perturb,
                                   &materialize, &adjoint, &loss_seed, &misfit_seed};
     return &t;

@@ -87,6 +87,30 @@ def test_two_steps_per_pass_d3q19(olb, name, dtype):
     _compare(CASES_3D[name][0](), dtype, (1, 2, 7), fused=True)
 
 
+# Several D2Q9 steps per launch (tiles of 64 x 32 cells with a halo of 8 or, on the
+# large lattices, 4): lattices below, at and just over a tile's part, smaller than a halo,
+# with force, porosity and TRT.
+CASES_2D = {
+    "box2x1": lambda: periodic_case(2, 1, 1, force=(1e-4, -2e-4, 0.0)),
+    "box2x3": lambda: periodic_case(2, 3, 1),
+    "box48x16": lambda: periodic_case(48, 16, 1),
+    "box50x17": lambda: periodic_case(50, 17, 1, force=(1e-4, -2e-4, 0.0)),
+    "box112x120": lambda: porous_box(112, 120, 1),
+    "trt": lambda: with_trt(periodic_case(96, 43, 1, force=(1e-4, -2e-4, 0.0))),
+}
+
+
+@pytest.mark.parametrize("dtype", ["f32", "f16", "bf16"])
+@pytest.mark.parametrize("name", sorted(CASES_2D))
+def test_several_steps_per_launch_d2q9(olb, name, dtype):
+    _compare(CASES_2D[name](), dtype, (1, 2, 5, 19), fused=True)
+
+
+@pytest.mark.parametrize("dtype,nx,ny", [("f32", 1100, 291), ("f16", 2002, 1990)])
+def test_several_steps_per_launch_d2q9_large(olb, dtype, nx, ny):
+    _compare(periodic_case(nx, ny, 1), dtype, (1, 2, 5, 19), fused=True)
+
+
 def _compare(case, dtype, counts, fused):
     import torch
 
