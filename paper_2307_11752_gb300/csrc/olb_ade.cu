@@ -24,6 +24,7 @@
 
 #include <cstdint>
 
+#include "olb_device.cuh"
 #include "olb_internal.h"
 
 namespace olb {
@@ -179,7 +180,7 @@ __global__ void __launch_bounds__(256) k_ade_density(AdeParams<T> p, const T* __
   if (c >= p.n) return;
   double s = 0.0;
 #pragma unroll
-  for (int i = 0; i < L::Q; ++i) s += (double)g[i * p.n + c];
+  for (int i = 0; i < L::Q; ++i) s += widen(g[i * p.n + c]);
   Cout[c] = s;
 }
 

@@ -82,19 +82,6 @@ inline bool pairs_ok(int) { return false; }
 inline bool pairs_ok(int nx) { return nx % 2 == 0; }
 #endif
 
-// n / d for 0 <= n < 2^31 by one high multiplication (T. Granlund, P. Montgomery,
-// "Division by invariant integers using multiplication", PLDI 1994).
-struct FastDiv {
-  unsigned d, m;
-  int s;
-  FastDiv() = default;
-  explicit FastDiv(unsigned d_) : d(d_), m(0), s(0) {
-    while ((1ull << s) < d) ++s;
-    m = (unsigned)(((1ull << (31 + s)) + d - 1) / d);
-  }
-  __device__ __forceinline__ unsigned div(unsigned n) const { return s == 0 ? n : __umulhi(n, m) >> (s - 1); }
-};
-
 // Launchers of one (lattice, storage type) pair.  Each returns the CUDA error of
 // the launch.  `partials` receives one row of 8 doubles per block (reductions).
 struct KernelTable {

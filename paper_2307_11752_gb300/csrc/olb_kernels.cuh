@@ -32,6 +32,7 @@
 #include <type_traits>
 #include <utility>
 
+#include "olb_device.cuh"
 #include "olb_internal.h"
 
 // The generic (one cell per thread) BGK collision with omega w_k folded into the
@@ -1014,7 +1015,7 @@ __global__ void __launch_bounds__(256) k_to_f64(Params<typename Store<S>::C> p, 
   C f[L::Q];
   gather<L, S, G>(p, src, n, cls, f);
 #pragma unroll
-  for (int i = 0; i < L::Q; ++i) out[i * N + n.cell] = (double)f[i] + L::w(i);
+  for (int i = 0; i < L::Q; ++i) out[i * N + n.cell] = widen(f[i]) + L::w(i);
 }
 
 template <class L, class S, int G>
@@ -1035,9 +1036,9 @@ __global__ void __launch_bounds__(256) k_moments(Params<typename Store<S>::C> p,
     moments<L>(f, drho, j);
     force_at(p, n.cell, F);
     const C rho = C(1) + drho;
-    r = (double)rho;
+    r = widen(rho);
 #pragma unroll
-    for (int d = 0; d < 3; ++d) u[d] = (double)((j[d] + C(0.5) * F[d]) / rho);
+    for (int d = 0; d < 3; ++d) u[d] = widen((j[d] + C(0.5) * F[d]) / rho);
   }
   if (rho_out) rho_out[n.cell] = r;
   if (u_out) {

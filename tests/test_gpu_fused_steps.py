@@ -111,6 +111,28 @@ def test_several_steps_per_launch_d2q9_large(olb, dtype, nx, ny):
     _compare(periodic_case(nx, ny, 1), dtype, (1, 2, 5, 19), fused=True)
 
 
+def test_populations_read_back_exactly(olb):
+    """Populations come back as (double)f + w for every FP32 pattern: zeros of both signs,
+    subnormals, the largest and smallest normals, infinities and NaN (D2Q9, whose
+    weights are added in FP64; stored values f - w are read through the rest weight)."""
+    import torch
+
+    bits = np.array([0, 0x80000000, 1, 0x80000001, 0x007fffff, 0x00800000, 0x80800000, 0x33d6bf95, 0x3f800000,
+                     0xbf7fffff, 0x7f7fffff, 0x7f800000, 0xff800000, 0x7fc00000], np.uint32)
+    v = bits.view(np.float32).astype(np.float64)
+    lat = olb.Lattice(olb.D2Q9, (len(v), 1, 1), dtype="f32")
+    lat.set_material(np.ones(len(v), np.uint8), 3)
+    w = 4.0 / 9.0
+    f = np.zeros((9, 1, 1, len(v)))
+    f[0, 0, 0] = v + w
+    lat.set_populations(torch.from_numpy(f).cuda())
+    got = lat.get_populations()[0, 0, 0].cpu().numpy()
+    with np.errstate(over="ignore"):
+        want = (f[0, 0, 0] - w).astype(np.float32).astype(np.float64) + w  # as stored, then widened
+    assert np.array_equal(got, want, equal_nan=True)
+    lat.close()
+
+
 def _compare(case, dtype, counts, fused):
     import torch
 
