@@ -33,6 +33,7 @@
 #include <utility>
 
 #include "olb_device.cuh"
+#include "olb_fold.h"
 #include "olb_internal.h"
 
 // The generic (one cell per thread) BGK collision with omega w_k folded into the
@@ -255,17 +256,6 @@ struct PairForce {
   float force[3], gs[9], ga[9], uf[2], src0;
 };
 
-// Constants of the FP64 collision (collide_folded), formed once on the host: on this GPU
-// an FP64 instruction of a warp holds an SM's FP64 pipe for 16 cycles, so products of
-// uniform values are not left to the threads.  Weight classes 0: rest, 1, 2: the moving
-// velocities (along an axis, diagonal).
-struct Fold64 {
-  double keep, even, odd;      // 1 - omega, (1 - omega)/2 and (1 - omega_odd)/2
-  double ow[3], b[3], t[3];    // omega w, 4.5 omega w, 3 omega_odd w
-  double gu[3];                // 3 (1 - omega/2) w
-  double gq[9], ga[9];         // 9 (1 - omega/2) w_k c_k.F,  3 (1 - omega_odd/2) w_k c_k.F
-};
-
 // Kernel parameters in the compute type C.
 template <class C>
 struct Params {
@@ -309,25 +299,14 @@ __host__ __device__ constexpr int weight_class(int k) {
 
 template <class L>
 Fold64 fold64(const Params<double>& p, bool trt) {
-  Fold64 r = {};
   const double odd = trt ? p.omega_minus : p.omega;
   const double ge = 1.0 - 0.5 * p.omega, go = 1.0 - 0.5 * odd;
-  r.keep = 1.0 - p.omega;
-  r.even = 0.5 * (1.0 - p.omega);
-  r.odd = 0.5 * (1.0 - odd);
-  for (int k = 0; k < L::Q; ++k) {
-    const int c = weight_class<L>(k);
-    const double w = L::w(k);
-    r.ow[c] = p.omega * w;
-    r.b[c] = 4.5 * p.omega * w;
-    r.t[c] = 3.0 * odd * w;
-    r.gu[c] = 3.0 * ge * w;
-    if (k > L::HALF) {
-      double cF = 0.0;
-      for (int a = 0; a < L::DIM; ++a) cF += L::c(k, a) * p.force[a];
-      r.gq[k - L::HALF - 1] = 9.0 * ge * w * cF;
-      r.ga[k - L::HALF - 1] = 3.0 * go * w * cF;
-    }
+  Fold64 r = fold64_rates(L::DIM, p.omega, odd);
+  for (int k = L::HALF + 1; k < L::Q; ++k) {
+    double cF = 0.0;
+    for (int a = 0; a < L::DIM; ++a) cF += L::c(k, a) * p.force[a];
+    r.gq[k - L::HALF - 1] = 9.0 * ge * L::w(k) * cF;
+    r.ga[k - L::HALF - 1] = 3.0 * go * L::w(k) * cF;
   }
   return r;
 }
@@ -664,9 +643,13 @@ __device__ __forceinline__ void collide(const Params<C>& p, C gamma, const C (&F
 //   TRT  f*_k, f*_opp = [(1 - omega)/2 (f_k + f_opp) + S] +- [(1 - omega_odd)/2 (f_k - f_opp) + A]
 // About 145 FP64 instructions on D3Q19 with or without force, where collide takes 250
 // with one.  The FP64 pipe bounds the step.
-template <class L, bool TRT>
-__device__ __forceinline__ void collide_folded(const Params<double>& p, double gamma, double (&f)[L::Q], double& drho,
-                                               double (&j)[3], double& rho, double (&u)[3]) {
+//
+// Without a force, rho u' is the momentum itself (times the porosity): A is formed from
+// it and S from it and 1/rho, so that the rounding of 1/rho does not reach the momentum
+// (where rho is within 1e-8 of 1, 1/rho rounds up more often than down).
+template <class L, bool TRT, bool FORCED>
+__device__ __forceinline__ void collide_folded_t(const Params<double>& p, double gamma, double (&f)[L::Q], double& drho,
+                                                 double (&j)[3], double& rho, double (&u)[3]) {
   const Fold64& c = p.fold;
   double s[L::HALF], a[L::HALF];
   drho = f[0];
@@ -690,42 +673,58 @@ __device__ __forceinline__ void collide_folded(const Params<double>& p, double g
   }
   rho = 1.0 + drho;
   const double inv = 1.0 / rho;
-  double up[3] = {0.0, 0.0, 0.0};
+  double q[3] = {0.0, 0.0, 0.0}, up[3] = {0.0, 0.0, 0.0};  // rho u' and u'
+  u[2] = 0.0;
 #pragma unroll
-  for (int d = 0; d < 3; ++d) u[d] = d < L::DIM ? (j[d] + p.half_force[d]) * inv : 0.0;
-#pragma unroll
-  for (int d = 0; d < L::DIM; ++d) up[d] = u[d];
+  for (int d = 0; d < L::DIM; ++d) {
+    q[d] = FORCED ? j[d] + p.half_force[d] : j[d];
+    u[d] = q[d] * inv;
+  }
   if (p.gamma) {
 #pragma unroll
-    for (int d = 0; d < L::DIM; ++d) up[d] = gamma * u[d];
+    for (int d = 0; d < L::DIM; ++d) q[d] *= gamma;
   }
+#pragma unroll
+  for (int d = 0; d < L::DIM; ++d) up[d] = q[d] * inv;
   double usq = up[0] * up[0] + up[1] * up[1];
   if (L::DIM == 3) usq += up[2] * up[2];
   const double dr = drho - 1.5 * rho * usq;
   double base[3] = {c.ow[0] * dr, c.ow[1] * dr, c.ow[2] * dr};
-  if (p.forced) {
+  if (FORCED) {
     double uF = up[0] * p.force[0] + up[1] * p.force[1];
     if (L::DIM == 3) uF += up[2] * p.force[2];
 #pragma unroll
     for (int k = 0; k < 3; ++k) base[k] -= c.gu[k] * uF;
   }
   f[0] = c.keep * f[0] + base[0];
-  const double br[3] = {0.0, c.b[1] * rho, c.b[2] * rho}, tr[3] = {0.0, c.t[1] * rho, c.t[2] * rho};
+  // c.v is c.u' with a force and rho c.u' without
+  double v[3], br[3], tr[3];
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    v[d] = FORCED ? up[d] : q[d];
+    br[d] = c.b[d] * (FORCED ? rho : inv);
+    tr[d] = FORCED ? c.t[d] * rho : c.t[d];
+  }
 #pragma unroll
   for (int k = 0; k < L::HALF; ++k) {
     const int kp = k + 1 + L::HALF, w = weight_class<L>(k + 1);
-    double cu = 0.0;
+    double cv = 0.0;
     bool first = true;
 #pragma unroll
     for (int d = 0; d < L::DIM; ++d) {
       if (L::c(kp, d) == 0) continue;
       if (first)
-        cu = L::c(kp, d) == 1 ? up[d] : -up[d];
+        cv = L::c(kp, d) == 1 ? v[d] : -v[d];
       else
-        cu = L::c(kp, d) == 1 ? cu + up[d] : cu - up[d];
+        cv = L::c(kp, d) == 1 ? cv + v[d] : cv - v[d];
       first = false;
     }
-    const double S = cu * (br[w] * cu + c.gq[k]) + base[w], A = tr[w] * cu + c.ga[k];
+    double S = br[w] * cv, A = tr[w] * cv;
+    if (FORCED) {
+      S += c.gq[k];
+      A += c.ga[k];
+    }
+    S = cv * S + base[w];
     if (TRT) {
       const double e = c.even * s[k] + S, o = c.odd * a[k] + A;
       f[kp] = e + o;
@@ -735,6 +734,15 @@ __device__ __forceinline__ void collide_folded(const Params<double>& p, double g
       f[k + 1] = c.keep * f[k + 1] + (S - A);
     }
   }
+}
+
+template <class L, bool TRT>
+__device__ __forceinline__ void collide_folded(const Params<double>& p, double gamma, double (&f)[L::Q], double& drho,
+                                               double (&j)[3], double& rho, double (&u)[3]) {
+  if (p.forced)
+    collide_folded_t<L, TRT, true>(p, gamma, f, drho, j, rho, u);
+  else
+    collide_folded_t<L, TRT, false>(p, gamma, f, drho, j, rho, u);
 }
 
 // ---------------------------------------------------------------------------------
