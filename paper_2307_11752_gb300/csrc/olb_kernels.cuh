@@ -179,6 +179,11 @@ constexpr int kWordMatShift = 22;
 // grid was launched without the attribute), so it comes before the first global
 // access; launch_dependents then allows the next step's grid to be scheduled
 // into the SM slots this grid's blocks free as they retire.
+//
+// Memory that an earlier launch may still be writing or reading (populations, adjoint
+// fields, the porosity and force fields) is passed without __restrict__: that qualifier
+// tells the compiler that nobody else touches the memory while the kernel runs, so it
+// could move an access above the wait, whose "memory" clobber does not cover it.
 __device__ __forceinline__ void pdl_wait() {
 #if OLB_PDL
   asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -273,8 +278,9 @@ struct Params {
   C domega_minus;  // TRT: d omega_minus / d omega at fixed magic parameter (BGK: 1)
   int forced;  // a uniform force or a force field is set
   // per-cell force density [3][ncell] in the compute type, or null (the uniform force)
-  const C* __restrict__ ffield;
-  const C* __restrict__ gamma;
+  // (filled by a kernel, so unqualified: see pdl_wait)
+  const C* ffield;
+  const C* gamma;
   // per cell: bit i set when x + c_i is a non-fluid cell of the lattice (a wall
   // link whose bounced population is stored in that cell)
   const uint32_t* __restrict__ pmask;
@@ -1210,8 +1216,8 @@ struct LambdaOf<double> {
 
 template <class L, class S, int G, bool TRT>
 __global__ void __launch_bounds__(256) k_adjoint(Params<typename Store<S>::C> p, const S* state,
-                                                 const typename LambdaOf<S>::T* __restrict__ lam_in,
-                                                 typename LambdaOf<S>::T* __restrict__ lam_out,
+                                                 const typename LambdaOf<S>::T* lam_in,
+                                                 typename LambdaOf<S>::T* lam_out,
                                                  double* dgamma, double* dforce, double* partials) {
   using C = typename Store<S>::C;
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1318,6 +1324,13 @@ __global__ void __launch_bounds__(256) k_adjoint(Params<typename Store<S>::C> p,
         base = om * (m0 + C(4.5) * um2u - C(1.5) * m0 * usq) + om_odd * C(3) * m1u - gi * Bu + direct;
       else
         base = om * A - gi * Bu + direct;
+      // read before the stores of lam_out, which the compiler must assume to overlap them
+      double dg = 0.0, dF[L::DIM];
+      if (dgamma) dg = dgamma[n.cell];
+      if (dforce) {
+#pragma unroll
+        for (int a = 0; a < L::DIM; ++a) dF[a] = dforce[(size_t)a * p.ncell + n.cell];
+      }
 #pragma unroll
       for (int i = 0; i < L::Q; ++i) {
         C Bc = C(0);
@@ -1336,7 +1349,7 @@ __global__ void __launch_bounds__(256) k_adjoint(Params<typename Store<S>::C> p,
         }
         lam_out[i * N + n.cell] = (typename LambdaOf<S>::T)(own + base + gi * Bc);
       }
-      if (dgamma) dgamma[n.cell] += (double)Bu;
+      if (dgamma) dgamma[n.cell] = dg + (double)Bu;
       if (dforce) {
         // through u = (j + F/2)/rho (B gamma / (2 rho)) and the Guo source's own F;
         // TRT: the source's odd part (m1) carries 1 - omega-/2
@@ -1344,8 +1357,8 @@ __global__ void __launch_bounds__(256) k_adjoint(Params<typename Store<S>::C> p,
         const C hg = C(0.5) * gi;
 #pragma unroll
         for (int a = 0; a < L::DIM; ++a)
-          dforce[(size_t)a * p.ncell + n.cell] +=
-              (double)(hg * B[a] + gf_odd * C(3) * m1[a] + gf * (C(9) * m2u[a] - C(3) * m0 * up[a]));
+          dforce[(size_t)a * p.ncell + n.cell] =
+              dF[a] + (double)(hg * B[a] + gf_odd * C(3) * m1[a] + gf * (C(9) * m2u[a] - C(3) * m0 * up[a]));
       }
       // dL/domega = sum_k lam*_k (feq_k - f_k) - G/2.  feq and f are both O(w) and
       // differ by the small non-equilibrium part, so the O(w) parts are removed

@@ -30,7 +30,7 @@ constexpr int kStripX = 64, kStripRows = 4, kStripWarps = 8, kStripY = kStripRow
 
 template <class S, bool TRT>
 __global__ void __launch_bounds__(32 * kStripWarps, 2)
-    k_strip(Params<float> p, const S* __restrict__ src, S* __restrict__ dst, StripGeom g) {
+    k_strip(Params<float> p, const S* src, S* dst, StripGeom g) {
   using L = D2Q9;
   using H = Held<S>;
   constexpr int R = kStripRows;
