@@ -398,7 +398,8 @@ int olb_ade_set_material(olb_ade_handle h, const uint8_t* material, unsigned per
 
 /* Advection velocity from a fluid lattice of the same size (D2Q9 for D2Q5, D3Q19
  * for D3Q7): v = u = (j + F/2)/rho of its current state, computed on the device
- * into this handle's velocity field (ordered after the fluid's queued work), so a
+ * into this handle's velocity field (ordered after the fluid's queued work, and before
+ * what is queued on the fluid afterwards, also where the two have different streams), so a
  * coupled step is olb_step(fluid, 1); olb_ade_set_velocity_from(h, fluid);
  * olb_ade_step(h, 1).  Errors: OLB_ERR_ARG (size or dimension mismatch). */
 int olb_ade_set_velocity_from(olb_ade_handle h, olb_handle fluid);

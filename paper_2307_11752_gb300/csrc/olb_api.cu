@@ -509,6 +509,18 @@ int input_view(olb_handle h, const void* p, size_t bytes, DevBuf& tmp, const voi
   return OLB_OK;
 }
 
+// Everything queued on `later` from here on waits for everything queued on `earlier`.
+int order_after(cudaStream_t later, cudaStream_t earlier) {
+  if (later == earlier) return OLB_OK;
+  cudaEvent_t ev;
+  OLB_CUDA(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming), "event");
+  cudaError_t e = cudaEventRecord(ev, earlier);
+  if (e == cudaSuccess) e = cudaStreamWaitEvent(later, ev, 0);
+  cudaEventDestroy(ev);
+  OLB_CUDA(e, "stream order");
+  return OLB_OK;
+}
+
 // Ensure the second population buffer exists.
 int ensure_other(olb_handle h) {
   DevBuf& b = h->buf[1 - h->cur];
@@ -1660,20 +1672,17 @@ int olb_ade_set_velocity_from(olb_ade_handle h, olb_handle fluid) {
     return fail(OLB_ERR_ARG, "the fluid lattice does not match the advection-diffusion lattice");
   const size_t bytes = 3 * (size_t)h->ncell * h->elem();
   if ((rc = h->vfield.reserve(bytes))) return rc;
-  // the fluid's state is final on its own stream; the moments run on this handle's
-  cudaEvent_t ev;
-  OLB_CUDA(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming), "event");
-  cudaError_t e = cudaEventRecord(ev, fluid->stream);
-  if (e == cudaSuccess) e = cudaStreamWaitEvent(h->stream, ev, 0);
-  cudaEventDestroy(ev);
-  OLB_CUDA(e, "stream order");
+  // the fluid's state is final on its own stream; the velocity is computed on this handle's
+  if ((rc = order_after(h->stream, fluid->stream))) return rc;
   HostParams p = fluid->params();
   p.stream = h->stream;
   OLB_CUDA(fluid->kt->velocity(p, gather_of(fluid->repr), fluid->buf[fluid->cur].p, h->vfield.p, h->dtype == OLB_F64),
            "fluid velocity");
   h->has_vfield = true;
   h->vfield_t = true;
-  return OLB_OK;
+  // and the fluid's later steps (in place with the AA pattern, into the other buffer and
+  // back with pull) write the populations only after they have been read
+  return order_after(fluid->stream, h->stream);
 }
 
 int olb_ade_init(olb_ade_handle h, const double* C) {
