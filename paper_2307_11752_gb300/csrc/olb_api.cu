@@ -1529,6 +1529,10 @@ int ade_input(olb_ade_handle h, const void* p, size_t bytes, DevBuf& tmp, const 
   return OLB_OK;
 }
 
+// The velocity field's buffer: one size for doubles and for the storage type, so that a
+// change from one form to the other neither frees what queued steps read nor can fail.
+int reserve_vfield(olb_ade_handle h) { return h->vfield.reserve(3 * (size_t)h->ncell * sizeof(double)); }
+
 }  // namespace
 
 extern "C" {
@@ -1599,7 +1603,7 @@ int olb_ade_set_velocity(olb_ade_handle h, const double v[3], const double* v_fi
   }
   if (v_field) {
     const size_t bytes = 3 * (size_t)h->ncell * sizeof(double);
-    if ((rc = h->vfield.reserve(bytes))) return rc;
+    if ((rc = reserve_vfield(h))) return rc;
     OLB_CUDA(cudaMemcpyAsync(h->vfield.p, v_field, bytes, cudaMemcpyDefault, h->stream), "velocity copy");
     OLB_CUDA(cudaStreamSynchronize(h->stream), "velocity sync");
     h->has_vfield = true;
@@ -1670,8 +1674,7 @@ int olb_ade_set_velocity_from(olb_ade_handle h, olb_handle fluid) {
   if ((rc = check(fluid))) return rc;
   if (fluid->nx != h->nx || fluid->ny != h->ny || fluid->nz != h->nz || fluid->dim != (h->q == 5 ? 2 : 3))
     return fail(OLB_ERR_ARG, "the fluid lattice does not match the advection-diffusion lattice");
-  const size_t bytes = 3 * (size_t)h->ncell * h->elem();
-  if ((rc = h->vfield.reserve(bytes))) return rc;
+  if ((rc = reserve_vfield(h))) return rc;
   // the fluid's state is final on its own stream; the velocity is computed on this handle's
   if ((rc = order_after(h->stream, fluid->stream))) return rc;
   HostParams p = fluid->params();
