@@ -733,6 +733,7 @@ int adjoint_sweep(olb_handle h, int64_t n_steps, int64_t K, Seed&& seed, double 
       const int g = srepr[k - 1] == PRE ? G_OWN : G_PULL;
       if (int e = launched(h, h->kt->step(h->params(), g, S_OWN, false, slot[k - 1], seg[k].p, nullptr), "recompute"))
         return e;
+      h->inject_tx = 0;  // an injection applies to one step
       slot[k] = seg[k].p;
       srepr[k] = POST;
     }
@@ -743,6 +744,7 @@ int adjoint_sweep(olb_handle h, int64_t n_steps, int64_t K, Seed&& seed, double 
     const int g = srepr[ks - 1] == PRE ? G_OWN : G_PULL;
     if (int e = launched(h, h->kt->step(h->params(), g, S_OWN, false, slot[ks - 1], h->buf[h->cur].p, nullptr), "step"))
       return e;
+    h->inject_tx = 0;
     h->repr = POST;
     h->time += ks;
     return (int)OLB_OK;
