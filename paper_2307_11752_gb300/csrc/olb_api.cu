@@ -723,7 +723,10 @@ int adjoint_sweep(olb_handle h, int64_t n_steps, int64_t K, Seed&& seed, double 
   const int saved_scheme = h->scheme;
   h->scheme = OLB_PULL;
   // The last segment steps through the segment's slots, so that the reverse sweep finds
-  // its states there: of n steps, n - K and not n are computed twice.
+  // its states there: of n steps in s segments of K, (s - 1)(K - 1) are computed twice
+  // instead of n - s.  Not on a lattice with halo planes: steps leave those alone, so the
+  // handle's own buffers hold what its steps read there, and the slots do not.
+  const bool keep_last = h->za <= 0 && h->zb >= h->nz - 1;
   std::vector<const void*> slot(K);
   std::vector<int> srepr(K);
   auto through_slots = [&](int64_t s, int64_t ks) {
@@ -753,11 +756,7 @@ int adjoint_sweep(olb_handle h, int64_t n_steps, int64_t K, Seed&& seed, double 
     OLB_CUDA(cudaMemcpyAsync(ckpt[s].p, h->buf[h->cur].p, sb, cudaMemcpyDeviceToDevice, h->stream), "checkpoint");
     ckpt_repr[s] = h->repr;
     const int64_t ks = std::min<int64_t>(K, n_steps - s * K);
-    if (s + 1 < nseg) {
-      rc = step_many(h, ks);
-    } else {
-      rc = last_segment(ks);
-    }
+    rc = keep_last && s + 1 == nseg ? last_segment(ks) : step_many(h, ks);
     if (rc) {
       h->scheme = saved_scheme;
       return rc;
@@ -781,7 +780,7 @@ int adjoint_sweep(olb_handle h, int64_t n_steps, int64_t K, Seed&& seed, double 
   int li = 0;
   for (int64_t s = nseg - 1; s >= 0; --s) {
     const int64_t ks = std::min<int64_t>(K, n_steps - s * K);
-    if (s + 1 < nseg && (rc = through_slots(s, ks))) return rc;
+    if (!(keep_last && s + 1 == nseg) && (rc = through_slots(s, ks))) return rc;
     for (int64_t k = ks - 1; k >= 0; --k) {
       const int g = srepr[k] == PRE ? G_OWN : G_PULL;
       if ((rc = launched(h, kt->adjoint(p, g, slot[k], lam[li].p, lam[1 - li].p, static_cast<double*>(dg.p),
