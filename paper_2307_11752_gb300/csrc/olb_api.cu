@@ -387,7 +387,6 @@ struct olb_lattice {
     p.err = static_cast<unsigned*>(err.p);
     p.inject_extra_tx = inject_tx;
     p.inject_wait_ns = (unsigned long long)inject_ns;
-    p.device = device;
     p.sms = sms;
     p.l2_bytes = l2_bytes;
     p.stream = stream;
@@ -607,25 +606,25 @@ int step_once(olb_handle h, bool stats, double* partials, int64_t* rows = nullpt
 // where the lattice allows it, else step by step.
 int step_many(olb_handle h, int64_t n) {
   int rc;
-  while (n > 0) {
-    if (n >= 2 && h->scheme == OLB_PULL && h->repr == POST && !h->inject_tx) {
-      const HostParams p = h->params();
-      const int strip = h->kt->strip_steps(p);
-      const int k = strip ? (int)std::min<int64_t>(strip, n) : (h->kt->step2_ok(p) ? 2 : 0);
-      if (k) {
-        if ((rc = ensure_other(h))) return rc;
-        const void* a = h->buf[h->cur].p;
-        void* b = h->buf[1 - h->cur].p;
-        if ((rc = launched(h, strip ? h->kt->strip(p, k, a, b) : h->kt->step2(p, a, b), "steps"))) return rc;
-        h->cur = 1 - h->cur;
-        h->time += k;
-        n -= k;
-        continue;
-      }
-    }
+  // up to the state after a pull step, from which several steps per launch start
+  while (n > 0 && !(n >= 2 && h->scheme == OLB_PULL && h->repr == POST && !h->inject_tx)) {
     if ((rc = step_once(h, false, nullptr))) return rc;
     --n;
   }
+  if (n > 0) {
+    const HostParams p = h->params();
+    const StepPlan plan = h->kt->plan(p);
+    while (n >= 2 && plan.per_launch() > 1) {
+      const int k = (int)std::min<int64_t>(plan.per_launch(), n);
+      if ((rc = ensure_other(h))) return rc;
+      if ((rc = launched(h, h->kt->steps(p, plan, k, h->buf[h->cur].p, h->buf[1 - h->cur].p), "steps"))) return rc;
+      h->cur = 1 - h->cur;
+      h->time += k;
+      n -= k;
+    }
+  }
+  for (; n > 0; --n)
+    if ((rc = step_once(h, false, nullptr))) return rc;
   return OLB_OK;
 }
 

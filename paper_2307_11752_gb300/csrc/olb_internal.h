@@ -51,8 +51,7 @@ struct HostParams {
   unsigned* err;          // device error word of the handle (set by kernels whose bounded waits ran out)
   unsigned inject_extra_tx;                // failure injection: bytes a TMA-fed step waits for beyond its copies
   unsigned long long inject_wait_ns;       // and the limit of its waits then
-  int device;             // the handle's device, its SM count and the bytes of its L2
-  int sms;
+  int sms;                // the device's SM count and the bytes of its L2
   int64_t l2_bytes;
   cudaStream_t stream;
 };
@@ -82,6 +81,35 @@ inline bool pairs_ok(int) { return false; }
 inline bool pairs_ok(int nx) { return nx % 2 == 0; }
 #endif
 
+// How a run of pull steps without statistics is cut into launches: `strip` steps per
+// launch (k_strip), or pairs of steps with `planes` planes per block (k_step2); both 0:
+// step by step.  Made once per call of olb_step and the like.
+struct StepPlan {
+  int strip = 0, planes = 0;
+  int per_launch() const { return strip ? strip : (planes ? 2 : 1); }
+};
+
+// The planes per block that give the fewest plane iterations on the SM with most blocks,
+// when nz planes of `tiles` tiles each are cut along z (a block needs 3 iterations more
+// than it has planes), and that number of iterations.  Only the sizes ceil(nz / n) are
+// looked at, each once: some 2 sqrt(nz) of them (7 us at nz = 65535 where all n take
+// 300).
+inline int64_t plane_split(int nz, int64_t tiles, int64_t sms, int& planes) {
+  int64_t best = INT64_MAX;
+  for (int c = nz; c >= 1;) {
+    const int n = (nz + c - 1) / c;
+    const int64_t cost = (tiles * n + sms - 1) / sms * (c + 3);
+    if (cost < best) {
+      best = cost;
+      planes = c;
+    }
+    if (c == 1) break;
+    const int next = (nz + c - 2) / (c - 1);  // the fewest blocks of fewer than c planes
+    c = (nz + next - 1) / next;
+  }
+  return best;
+}
+
 // Launchers of one (lattice, storage type) pair.  Each returns the CUDA error of
 // the launch.  `partials` receives one row of 8 doubles per block (reductions).
 struct KernelTable {
@@ -92,12 +120,10 @@ struct KernelTable {
                       void* dst, double* partials);
   // rows of partial sums that step() with these patterns writes when stats is set
   int64_t (*step_rows)(const HostParams&, int gather, int scatter);
-  // two pull steps from a POST state to a POST state in one pass, where the lattice allows it
-  bool (*step2_ok)(const HostParams&);
-  cudaError_t (*step2)(const HostParams&, const void* src, void* dst);
-  // n <= strip_steps() pull steps (0: not offered) from a POST state to a POST state in one launch
-  int (*strip_steps)(const HostParams&);
-  cudaError_t (*strip)(const HostParams&, int n, const void* src, void* dst);
+  // several pull steps from a POST state to a POST state per launch, where the lattice
+  // allows it: n <= plan.per_launch() steps (n == 2 where plan.planes is set)
+  StepPlan (*plan)(const HostParams&);
+  cudaError_t (*steps)(const HostParams&, const StepPlan& plan, int n, const void* src, void* dst);
   cudaError_t (*to_f64)(const HostParams&, int gather, const void* src, double* f);
   cudaError_t (*moments)(const HostParams&, int gather, const void* src, double* rho, double* u);
   // the velocity alone, [3][cells] in double or float

@@ -28,7 +28,6 @@
 #include <cuda_fp16.h>
 #include <stdint.h>
 
-#include <atomic>
 #include <type_traits>
 #include <utility>
 
@@ -1731,26 +1730,13 @@ struct Launch {
     return launch_step(k_step<L, S, G, SC, STATS, TRT>, g.dims(), dim3(256), 0, h.stream, params(h),
                        static_cast<const S*>(src), static_cast<S*>(dst), partials);
   }
-  // Tiles of the two-step pass (k_step2) and the planes per block that give the fewest
-  // plane iterations on the SM with most blocks.
-  static int64_t step2_geometry(const HostParams& h, int& xt, int& yt, int& cz) {
-    using M = March<S>;
-    const int nz = h.z1 - h.z0 + 1;
-    xt = (h.nx + M::TX - 1) / M::TX;
-    yt = (h.y1 - h.y0 + M::TY) / M::TY;
-    int64_t cost = INT64_MAX;
-    for (int nc = 1; nc <= nz; ++nc) {
-      const int c = (nz + nc - 1) / nc;
-      const int64_t waves = ((int64_t)xt * yt * ((nz + c - 1) / c) + h.sms - 1) / h.sms;
-      if (waves * (c + 3) < cost) {
-        cost = waves * (c + 3);
-        cz = c;
-      }
-    }
-    return cost;
-  }
 
-  // Whether two pull steps from a POST state run as one pass (k_step2).  It accepts
+  // Tiles of the two-step pass (k_step2).
+  static int step2_xt(const HostParams& h) { return (h.nx + March<S>::TX - 1) / March<S>::TX; }
+  static int step2_yt(const HostParams& h) { return (h.y1 - h.y0 + March<S>::TY) / March<S>::TY; }
+
+  // Planes per block when two pull steps from a POST state run as one pass (k_step2), 0
+  // when they do not.  It accepts
   // lattices with a uniform or no force and no link that leaves the domain, nx even,
   // and pays where single steps are bound by HBM: both buffers together beyond L2.
   // A plane iteration costs 3.5 to 4.0 us without and 4.8 us with walls on all SMs at
@@ -1763,44 +1749,38 @@ struct Launch {
   // from four times L2.  The Guo source adds a quarter to the arithmetic
   // (channel 128^3 50.2 -> 49.0 us, TRT 97.4 -> 96.5 us: not worth the state), so
   // forced lattices step one by one.
-  static bool step2_ok(const HostParams& h) {
+  static int step2_planes(const HostParams& h) {
     if constexpr (std::is_same<S, double>::value || L::DIM != 3) {
-      return false;
+      return 0;
     } else {
       const bool walls = h.cls != nullptr;
       if (!pairs_ok(h.nx) || h.ffield != nullptr || h.forced || h.outside_links || h.az0 != 0 || h.az1 != h.nz - 1 ||
           tma_setting("OLB_TMA", OLB_TMA))
-        return false;
-      if (sizeof(S) == 2 && walls) return false;
+        return 0;
+      if (sizeof(S) == 2 && walls) return 0;
       const uint64_t plane_bytes = (uint64_t)h.pitch * sizeof(S);
-      if (plane_bytes >= (1ull << 32) || (uint64_t)h.nx * h.ny * sizeof(S) >= (1ull << 31)) return false;  // k_step2
-      if (2 * L::Q * plane_bytes <= (sizeof(S) == 2 ? 4 : 1) * (uint64_t)h.l2_bytes) return false;
-      int xt, yt, cz;
-      const int64_t planes = step2_geometry(h, xt, yt, cz);
+      if (plane_bytes >= (1ull << 32) || (uint64_t)h.nx * h.ny * sizeof(S) >= (1ull << 31)) return 0;  // k_step2
+      if (2 * L::Q * plane_bytes <= (sizeof(S) == 2 ? 4 : 1) * (uint64_t)h.l2_bytes) return 0;
+      int planes = 0;
+      const int64_t n = plane_split(h.z1 - h.z0 + 1, (int64_t)step2_xt(h) * step2_yt(h), h.sms, planes);
       const double cells = (double)h.nx * (h.y1 - h.y0 + 1) * (h.z1 - h.z0 + 1);
-      return cells > (walls ? 0.72 : 0.66) * (double)planes * h.sms * (March<S>::TX * March<S>::TY);
+      return cells > (walls ? 0.72 : 0.66) * (double)n * h.sms * (March<S>::TX * March<S>::TY) ? planes : 0;
     }
   }
 
   template <bool WALLS, bool TRT>
-  static cudaError_t launch_step2(const HostParams& h, const void* src, void* dst) {
+  static cudaError_t launch_step2(const HostParams& h, int planes, const void* src, void* dst) {
     using M = March<S>;
     auto kernel = k_step2<S, WALLS, TRT>;
-    // shared memory above 48 KB is granted once per device
-    static std::atomic<uint64_t> granted{0};
-    const uint64_t bit = uint64_t(1) << (h.device & 63);
-    if (!(granted.load(std::memory_order_relaxed) & bit)) {
-      cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)M::smem());
-      if (e != cudaSuccess) return e;
-      granted.fetch_or(bit, std::memory_order_relaxed);
-    }
+    // shared memory above 48 KB; granted at each launch (under 1 us beside a kernel of 80
+    // and more), since a grant ends with its context
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)M::smem());
+    if (e != cudaSuccess) return e;
     const Params<float> p = params(h);
     const MarchBuf<S> pl{static_cast<const S*>(src), static_cast<S*>(dst), (unsigned)(h.pitch * sizeof(S))};
-    int xt, yt, cz;
-    step2_geometry(h, xt, yt, cz);
     const int nz = h.z1 - h.z0 + 1;
-    return launch_step(kernel, dim3(xt, yt, (nz + cz - 1) / cz), dim3(M::THREADS), M::smem(), h.stream, p, pl,
-                       MarchGeom{cz});
+    return launch_step(kernel, dim3(step2_xt(h), step2_yt(h), (nz + planes - 1) / planes), dim3(M::THREADS), M::smem(),
+                       h.stream, p, pl, MarchGeom{planes});
   }
 
   // Steps that one launch of k_strip takes (0: the lattice has no such path).  Halo 8
@@ -1823,29 +1803,31 @@ struct Launch {
     }
   }
 
-  // n <= strip_steps(h) pull steps, POST to POST.
-  static cudaError_t strip(const HostParams& h, int n, const void* src, void* dst) {
-    if constexpr (std::is_same<S, double>::value || L::DIM != 2) {
+  static StepPlan plan(const HostParams& h) {
+    StepPlan r;
+    r.strip = strip_steps(h);
+    if (!r.strip) r.planes = step2_planes(h);
+    return r;
+  }
+
+  // n pull steps in one launch by plan(h), POST to POST.
+  static cudaError_t steps(const HostParams& h, const StepPlan& plan, int n, const void* src, void* dst) {
+    if constexpr (std::is_same<S, double>::value) {
       return cudaErrorNotSupported;
-    } else {
-      const StripGeom g{strip_steps(h), n};
+    } else if constexpr (L::DIM == 2) {
+      const StripGeom g{plan.strip, n};
       const int ow = kStripX - 2 * g.halo, oh = kStripY - 2 * g.halo;
       const dim3 grid((h.nx + ow - 1) / ow, (h.ny + oh - 1) / oh), block(32 * kStripWarps);
       return launch_step(h.trt ? k_strip<S, true> : k_strip<S, false>, grid, block, 0, h.stream, params(h),
                          static_cast<const S*>(src), static_cast<S*>(dst), g);
-    }
-  }
-
-  // Two pull steps, POST to POST.
-  static cudaError_t step2(const HostParams& h, const void* src, void* dst) {
-    if constexpr (std::is_same<S, double>::value || L::DIM != 3) {
-      return cudaErrorNotSupported;
     } else {
       if constexpr (sizeof(S) == 4) {
         if (h.cls != nullptr)
-          return h.trt ? launch_step2<true, true>(h, src, dst) : launch_step2<true, false>(h, src, dst);
+          return h.trt ? launch_step2<true, true>(h, plan.planes, src, dst)
+                       : launch_step2<true, false>(h, plan.planes, src, dst);
       }
-      return h.trt ? launch_step2<false, true>(h, src, dst) : launch_step2<false, false>(h, src, dst);
+      return h.trt ? launch_step2<false, true>(h, plan.planes, src, dst)
+                   : launch_step2<false, false>(h, plan.planes, src, dst);
     }
   }
 
@@ -1966,7 +1948,7 @@ struct Launch {
   }
 
   static const KernelTable* table() {
-    static const KernelTable t = {L::Q,       sizeof(S), sizeof(T), &step,    &step_rows, &step2_ok, &step2, &strip_steps, &strip, &to_f64,
+    static const KernelTable t = {L::Q,       sizeof(S), sizeof(T), &step,    &step_rows, &plan, &steps, &to_f64,
                                   &moments,   &velocity,  &stats,    &from_f64, &init_eq, &perturb,
                                   &materialize, &adjoint, &loss_seed, &misfit_seed};
     return &t;
