@@ -182,7 +182,10 @@ int olb_perturb_populations(olb_handle h, const double* df);
 int olb_set_populations(olb_handle h, const double* f);
 int olb_get_populations(olb_handle h, double* f);
 
-/* Advance the state by n >= 0 collide-and-stream steps (asynchronous). */
+/* Advance the state by n >= 0 collide-and-stream steps (asynchronous).  A stream
+ * capture of an even n (from a state that a step has left, so that nothing is allocated)
+ * gives a graph each replay of which advances the state by n; the time counter counts
+ * the call, not the replays. */
 int olb_step(olb_handle h, int64_t n);
 
 /* Advance by n >= 1 steps like olb_step and return the lattice statistics that

@@ -602,8 +602,20 @@ int step_once(olb_handle h, bool stats, double* partials, int64_t* rows = nullpt
   return OLB_OK;
 }
 
+// Whether the handle's stream is being captured into a graph.
+bool capturing(olb_handle h) {
+  cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(h->stream, &s) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return s != cudaStreamCaptureStatusNone;
+}
+
 // n steps in the handle's scheme without statistics: several pull steps per launch
-// where the lattice allows it, else step by step.
+// where the lattice allows it, else step by step.  Under stream capture always step by
+// step: a graph of an even number of steps then ends in the buffer that it started from,
+// so that each replay goes on from the one before.
 int step_many(olb_handle h, int64_t n) {
   int rc;
   // up to the state after a pull step, from which several steps per launch start
@@ -613,7 +625,7 @@ int step_many(olb_handle h, int64_t n) {
   }
   if (n > 0) {
     const HostParams p = h->params();
-    const StepPlan plan = h->kt->plan(p);
+    const StepPlan plan = capturing(h) ? StepPlan() : h->kt->plan(p);
     while (n >= 2 && plan.per_launch() > 1) {
       const int k = (int)std::min<int64_t>(plan.per_launch(), n);
       if ((rc = ensure_other(h))) return rc;
