@@ -136,16 +136,20 @@ def measured_peak_gbs():
 
 
 def kernel_source_sha():
+    """Hash of every header of the kernels (a step may run any of them)."""
     h = hashlib.sha256()
-    for rel in ("paper_2307_11752_gb300/csrc/olb_kernels.cuh", "paper_2307_11752_gb300/csrc/olb_pair.cuh"):
-        with open(os.path.join(ROOT, rel), "rb") as fh:
-            h.update(fh.read())
+    csrc = os.path.join(ROOT, "paper_2307_11752_gb300", "csrc")
+    for name in sorted(os.listdir(csrc)):
+        if name.endswith((".cuh", ".h")):
+            with open(os.path.join(csrc, name), "rb") as fh:
+                h.update(name.encode() + b"\0" + fh.read())
     return h.hexdigest()[:16]
 
 
-def profiled_traffic(kernel_key: str, units: int):
+def profiled_traffic(kernel_key: str, units: int, steps_per_launch: float):
     """DRAM bytes per launch of the step kernel from the committed ncu summary, scaled
-    to `units` fluid cells; None when the kernel source changed since the capture."""
+    to `units` fluid cells; None when the kernel source changed since the capture or the
+    captured launches advanced by another number of steps than the timed ones."""
     try:
         with open(PROFILE_TRAFFIC) as fh:
             rec = json.load(fh)
@@ -153,6 +157,8 @@ def profiled_traffic(kernel_key: str, units: int):
         return None
     entry = rec.get(kernel_key)
     if not entry or entry.get("source_sha") != kernel_source_sha():
+        return None
+    if entry.get("steps_per_launch", 1) != round(steps_per_launch, 1):
         return None
     return float(entry["dram_bytes_per_fluid_cell"]) * units
 
@@ -259,7 +265,7 @@ def variants(olb, torch):
         out[key] = {
             "MLUPS": round(fluid / ms / 1e3, 1), "bytes_per_update": b, "steps_per_launch": round(per, 2),
             "roofline_frac": round(fluid * b / (per * ms * 1e-3) / 1e9 / peak, 4)}
-        traffic = profiled_traffic(key, fluid)
+        traffic = profiled_traffic(key, fluid, per)
         if traffic is not None:
             out[key]["traffic"] = round(traffic)  # DRAM bytes per launch (ncu), mean over the pattern's launches
         lat.close()
@@ -274,7 +280,7 @@ def variants(olb, torch):
         out[key] = {
             "MLUPS": round(fluid / ms / 1e3, 1), "bytes_per_update": b, "steps_per_launch": round(per, 2),
             "roofline_frac": round(fluid * b / (per * ms * 1e-3) / 1e9 / peak, 4)}
-        traffic = profiled_traffic(key, fluid)
+        traffic = profiled_traffic(key, fluid, per)
         if traffic is not None:
             out[key]["traffic"] = round(traffic)
         lat.close()
@@ -671,7 +677,7 @@ def run_ours(args):
     peak, peak_kind = measured_peak_gbs()
     bytes_per_launch = fluid * 152
     achieved = bytes_per_launch / (kernel_ms * 1e-3) / 1e9
-    traffic = profiled_traffic("cavity128_f32_pull", fluid)
+    traffic = profiled_traffic("cavity128_f32_pull", fluid, per_launch)
     e2e_units = fluid * LBM_STEPS * max(1, min(args.steps, 3)) * world
     extra = variants(olb, torch) if (args.variants and rank == 0) else None
     if world > 1:
