@@ -227,14 +227,14 @@ __device__ __forceinline__ void collide_pair_t(const Params<float>& p, F2 gamma,
   const F2 T = F2(3.0f) * rho;
   F2 uF(0.0f);
   if (FORCED) {
-    uF = up[0] * F2(p.pf.force[0]);
-    uF = fma2(up[1], F2(p.pf.force[1]), uF);
-    uF = fma2(up[2], F2(p.pf.force[2]), uF);
+    uF = up[0] * F2(p.t.pf.force[0]);
+    uF = fma2(up[1], F2(p.t.pf.force[1]), uF);
+    uF = fma2(up[2], F2(p.t.pf.force[2]), uF);
   }
   {
     const float w0 = (float)L::w(0);
     F2 v = fma2(one_m_om, f[0], F2(om * w0) * A);
-    if (FORCED) v = fma2(F2(p.pf.src0), uF, v);
+    if (FORCED) v = fma2(F2(p.t.pf.src0), uF, v);
     f[0] = v;
   }
 #pragma unroll
@@ -272,8 +272,8 @@ __device__ __forceinline__ void collide_pair_t(const Params<float>& p, F2 gamma,
     }
     if (FORCED) {
       // Guo: gf w (9 cu cF - 3 u'.F) +- 3 gf w cF   (F in scaled units)
-      const F2 gs = fma2(F2(p.pf.gs[k - 1]), cu, F2(wk == (float)L::w(1) ? p.pf.uf[0] : p.pf.uf[1]) * uF);
-      const F2 ga(p.pf.ga[k - 1]);
+      const F2 gs = fma2(F2(p.t.pf.gs[k - 1]), cu, F2(wk == (float)L::w(1) ? p.t.pf.uf[0] : p.t.pf.uf[1]) * uF);
+      const F2 ga(p.t.pf.ga[k - 1]);
       fp = fp + gs + ga;
       fm = fm + gs - ga;
     }
