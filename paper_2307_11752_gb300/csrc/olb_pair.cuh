@@ -168,13 +168,16 @@ __device__ __forceinline__ void st_pair(S* plane, const PairNbr& n, int dx, int 
 // Returns rho_s and u for the wall terms and statistics.
 // ---------------------------------------------------------------------------------
 // TRT = true: the two-relaxation-time operator (see collide in olb_kernels.cuh).
-// FORCED: the Guo source with the uniform force; its constants per direction come
-// from the host (PairForce), already as pairs, instead of from ~75 scalar
-// multiplications per pair of cells.
-template <class L, int SCALE_NUM, bool TRT, bool FORCED>
+// FORCE: without (kForceNone) or with (kForceGuo) the Guo source of the uniform force,
+// or as p.forced says (kForceRuntime); its constants per direction come from the host
+// (PairForce), already as pairs, instead of from ~75 scalar multiplications per pair of
+// cells.
+enum PairForceMode { kForceNone = 0, kForceGuo = 1, kForceRuntime = 2 };
+template <class L, int SCALE_NUM, bool TRT, int FORCE>
 __device__ __forceinline__ void collide_pair_t(const Params<float>& p, F2 gamma, F2 (&f)[L::Q], F2& drho_s,
                                                F2 (&j_s)[3], F2& rho_s, F2 (&u)[3]) {
   constexpr float SCALE = (float)SCALE_NUM;
+  const bool forced = FORCE == kForceRuntime ? p.forced != 0 : FORCE == kForceGuo;
   // moments
   F2 d = f[0];
   F2 jj[3];
@@ -208,7 +211,7 @@ __device__ __forceinline__ void collide_pair_t(const Params<float>& p, F2 gamma,
   F2 up[3];
 #pragma unroll
   for (int dd = 0; dd < 3; ++dd) {
-    u[dd] = (FORCED ? jj[dd] + F2(p.half_force[dd] * SCALE) : jj[dd]) * inv;
+    u[dd] = (forced ? jj[dd] + F2(p.half_force[dd] * SCALE) : jj[dd]) * inv;
     up[dd] = u[dd];
   }
   if (p.gamma) {
@@ -226,7 +229,7 @@ __device__ __forceinline__ void collide_pair_t(const Params<float>& p, F2 gamma,
   const F2 B = F2(4.5f) * rho;
   const F2 T = F2(3.0f) * rho;
   F2 uF(0.0f);
-  if (FORCED) {
+  if (forced) {
     uF = up[0] * F2(p.t.pf.force[0]);
     uF = fma2(up[1], F2(p.t.pf.force[1]), uF);
     uF = fma2(up[2], F2(p.t.pf.force[2]), uF);
@@ -234,7 +237,7 @@ __device__ __forceinline__ void collide_pair_t(const Params<float>& p, F2 gamma,
   {
     const float w0 = (float)L::w(0);
     F2 v = fma2(one_m_om, f[0], F2(om * w0) * A);
-    if (FORCED) v = fma2(F2(p.t.pf.src0), uF, v);
+    if (forced) v = fma2(F2(p.t.pf.src0), uF, v);
     f[0] = v;
   }
 #pragma unroll
@@ -270,7 +273,7 @@ __device__ __forceinline__ void collide_pair_t(const Params<float>& p, F2 gamma,
       fp = f[kp] - (even + odd);
       fm = f[k] - (even - odd);
     }
-    if (FORCED) {
+    if (forced) {
       // Guo: gf w (9 cu cF - 3 u'.F) +- 3 gf w cF   (F in scaled units)
       const F2 gs = fma2(F2(p.t.pf.gs[k - 1]), cu, F2(wk == (float)L::w(1) ? p.t.pf.uf[0] : p.t.pf.uf[1]) * uF);
       const F2 ga(p.t.pf.ga[k - 1]);
@@ -282,13 +285,20 @@ __device__ __forceinline__ void collide_pair_t(const Params<float>& p, F2 gamma,
   }
 }
 
-template <class L, int SCALE_NUM, bool TRT = false>
+// One instance without and one with the force behind one branch (128^3 FP32 box, AA 50.5
+// -> 49.3 us a half step), or INLINE_FORCE: one instance that asks at each use.  In 3D that
+// suits the FP32 AA half steps with walls, where registers are short (128^3 cavity 56.8 ->
+// 55.7 us), and the BGK pull step without walls (128^3 box FP16 28.6 -> 27.9, FP32 47.7 ->
+// 47.6).  In 2D it does not (1024^2 cavity FP32 AA 10.5 -> 11.0, FP16 pull 9.68 -> 9.76).
+template <class L, int SCALE_NUM, bool TRT = false, bool INLINE_FORCE = false>
 __device__ __forceinline__ void collide_pair(const Params<float>& p, F2 gamma, F2 (&f)[L::Q], F2& drho_s,
                                              F2 (&j_s)[3], F2& rho_s, F2 (&u)[3]) {
-  if (p.forced)
-    collide_pair_t<L, SCALE_NUM, TRT, true>(p, gamma, f, drho_s, j_s, rho_s, u);
+  if (INLINE_FORCE)
+    collide_pair_t<L, SCALE_NUM, TRT, kForceRuntime>(p, gamma, f, drho_s, j_s, rho_s, u);
+  else if (p.forced)
+    collide_pair_t<L, SCALE_NUM, TRT, kForceGuo>(p, gamma, f, drho_s, j_s, rho_s, u);
   else
-    collide_pair_t<L, SCALE_NUM, TRT, false>(p, gamma, f, drho_s, j_s, rho_s, u);
+    collide_pair_t<L, SCALE_NUM, TRT, kForceNone>(p, gamma, f, drho_s, j_s, rho_s, u);
 }
 
 // 6 w_i (c_i . u_w) of wall material m (FP32 table).
@@ -427,7 +437,9 @@ __device__ __forceinline__ void pair_update(const Params<float>& p, const P& pl,
     }
   }
   F2 drho, j[3], rho, u[3];
-  collide_pair<L, SC_NUM, TRT>(p, gamma, f, drho, j, rho, u);
+  // (see collide_pair)
+  constexpr bool INLINE_FORCE = L::DIM == 3 && (WALLS ? sizeof(S) == 4 && SC != S_OWN : SC == S_OWN && !TRT);
+  collide_pair<L, SC_NUM, TRT, INLINE_FORCE>(p, gamma, f, drho, j, rho, u);
   const bool fl0 = (w[0] & kWordFluid) != 0, fl1 = (w[1] & kWordFluid) != 0;
   if (!WALLS) {
     // every cell fluid, every axis periodic: plain paired stores only
