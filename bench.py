@@ -590,8 +590,8 @@ def experiment_domain_id(torch, olb, dtype="f32", iterations=20):
     return out
 
 
-PROFILE_CASES = ("cavity128_{f32,f16,bf16}_{pull,aa}[_trt], tgv256_{f32,f16}_pull, "
-                 "adjoint_channel128_f32")
+PROFILE_CASES = ("cavity128_{f32,f16,bf16,f64}_{pull,aa}[_trt], tgv256_{f32,f16}_pull, "
+                 "box2d2048_{f32,f16}_pull, adjoint_channel128_f32")
 
 
 def run_profile_case(torch, olb, case: str, launches: int):
@@ -615,6 +615,13 @@ def run_profile_case(torch, olb, case: str, launches: int):
         rho, u = I.tgv3d(n, 0.02, xp=torch, device="cuda")
         lat.init_equilibrium(rho.reshape(-1), u.reshape(-1))
         del rho, u
+        lat.step(launches)
+    elif parts[0] == "box2d2048":
+        n = 2048
+        lat = olb.Lattice(olb.D2Q9, (n, n, 1), dtype=parts[1], scheme=parts[2])
+        lat.set_material(torch.ones(n * n, dtype=torch.uint8, device="cuda"), 3)
+        lat.set_bgk(0.6)
+        lat.init_equilibrium()
         lat.step(launches)
     elif case == "adjoint_channel128_f32":
         lat, m = porous_channel(olb, torch, 128, 64, 64, "f32")

@@ -221,7 +221,8 @@ typedef struct {
 /* Run n_steps steps from the current state, evaluate the objective L on the final
  * state, and return dL/dgamma (double [cells], 0 on non-fluid cells) and dL/dtau.
  * Forward states are checkpointed every `checkpoint_every` steps and each segment
- * is recomputed in reverse before its adjoint steps.  The handle ends in the final
+ * but the last (whose states are kept; with halo planes the last too) is recomputed in
+ * reverse before its adjoint steps.  The handle ends in the final
  * forward state (time advanced by n_steps), as after olb_step(h, n_steps).
  * The gradient is with respect to the porosity field set by olb_set_porosity
  * (gamma = 1 everywhere when none is set).  Any of loss, dL_dgamma, dL_dtau may

@@ -36,8 +36,9 @@
 #include "olb_internal.h"
 
 // The generic (one cell per thread) BGK collision with omega w_k folded into the
-// equilibrium's coefficients per weight class: fewer arithmetic instructions, which
-// is what bounds the FP64 step on this GPU.
+// equilibrium's coefficients per weight class: fewer arithmetic instructions.  FP32 and
+// 16-bit lattices with odd nx or a force field run it, and FP64 ones with a force field
+// (FP64 without one: collide_folded).
 #ifndef OLB_FOLD_OMEGA_GENERIC
 #define OLB_FOLD_OMEGA_GENERIC 1
 #endif
@@ -660,8 +661,9 @@ __device__ __forceinline__ void collide(const Params<C>& p, C gamma, const C (&F
 //   A = 3 omega_odd w rho c.u' + 3 go w c.F      (ge = 1 - omega/2, go = 1 - omega_odd/2)
 //   BGK  f*_k = (1 - omega) f_k + (S + A),  f*_opp = (1 - omega) f_opp + (S - A)
 //   TRT  f*_k, f*_opp = [(1 - omega)/2 (f_k + f_opp) + S] +- [(1 - omega_odd)/2 (f_k - f_opp) + A]
-// About 145 FP64 instructions on D3Q19 with or without force, where collide takes 250
-// with one.  The FP64 pipe bounds the step.
+// About 145 FP64 instructions on D3Q19 with a force, where collide takes 250; 64^2 D2Q9
+// vortex (no force) 3.8 -> 3.5 us a step with an instance of its own.  The FP64 pipe bounds
+// the step.
 //
 // Without a force, rho u' is the momentum itself (times the porosity): A is formed from
 // it and S from it and 1/rho, so that the rounding of 1/rho does not reach the momentum
@@ -938,7 +940,7 @@ __device__ __forceinline__ bool on_edge(const Params<C>& p, int x, int y, int z)
 // FP64: cells are dealt to the threads by a flat index over the rows that hold fluid, so
 // that warps are full at any nx (75 cells a row: 78 % of the lanes in rows of 32), in
 // blocks small enough to reach every SM on small lattices (flat_threads).
-// 75x61x57 channel with force: 152 -> 72 us; 64^2 D2Q9 vortex: 7.9 -> 3.8 us a step.
+// 75x61x57 channel with force: 152 -> 72 us; 64^2 D2Q9 vortex: 7.9 -> 3.5 us a step.
 template <class L, class S, int G, int SC, bool STATS, bool TRT>
 __global__ void __launch_bounds__(std::is_same<S, double>::value ? 128 : 256,
                                   std::is_same<S, double>::value ? 4 : OLB_STEP_MIN_BLOCKS)

@@ -5,9 +5,10 @@
 // A 2D step moves 72 bytes a cell (FP32) through L2 or, from about 1400^2, HBM, and a
 // small one waits for its launch.  Here a block loads a tile of 64 x 32 cells once,
 // advances it by up to `halo` steps and stores the cells that are still valid: one ring
-// of cells is lost per step.  The tiles' overlap is redundant arithmetic (1.3 times the
-// cells at halo 4, 1.9 at halo 8), which pays against the traffic of a large lattice
-// and the launches of a small one: 2048^2 FP32 45.9 -> 28.9 us a step, 64^2 2.07 -> 1.59.
+// of cells is lost per step.  Every step collides the whole tile: 2048 cells for the 1344
+// that are stored at halo 4 (1.5 times the arithmetic), for 768 at halo 8 (2.7 times).
+// That pays against the traffic of a large lattice and the launches of a small one:
+// 2048^2 FP32 45.9 -> 28.9 us a step, 64^2 2.07 -> 1.59.
 // (The same with walls needs their links in every step: 1024^2 cavity 10.9 -> 13.8 us,
 // 511 x 213 with an obstacle 3.1 -> 4.4; those lattices step one by one.)
 //
