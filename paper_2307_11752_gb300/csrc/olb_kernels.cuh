@@ -1234,8 +1234,12 @@ struct LambdaOf<double> {
   using T = double;
 };
 
-template <class L, class S, int G, bool TRT>
-__global__ void __launch_bounds__(256) k_adjoint(Params<typename Store<S>::C> p, const S* state,
+// BLOCKS: blocks per SM that it is compiled for, 0 for what the compiler takes: 80
+// registers in the BGK instances of FP32 arithmetic, three blocks per SM.  At 4 (64
+// registers) lattices of more blocks than that are faster and smaller ones slower: rule
+// and figures in adjoint_t.
+template <class L, class S, int G, bool TRT, int BLOCKS>
+__global__ void __launch_bounds__(256, BLOCKS) k_adjoint(Params<typename Store<S>::C> p, const S* state,
                                                  const typename LambdaOf<S>::T* lam_in,
                                                  typename LambdaOf<S>::T* lam_out,
                                                  double* dgamma, double* dforce, double* partials) {
@@ -1938,12 +1942,20 @@ struct Launch {
     const T* li = static_cast<const T*>(lam_in);
     T* lo = static_cast<T*>(lam_out);
     if (gather == G_OWN)
-      return launch_step(k_adjoint<L, S, G_OWN, TRT>, g.grid, g.block, 0, h.stream, params(h), st, li, lo, dgamma,
+      return launch_step(k_adjoint<L, S, G_OWN, TRT, 0>, g.grid, g.block, 0, h.stream, params(h), st, li, lo, dgamma,
                          dforce, partials);
-    if (gather == G_PULL)
-      return launch_step(k_adjoint<L, S, G_PULL, TRT>, g.grid, g.block, 0, h.stream, params(h), st, li, lo, dgamma,
-                         dforce, partials);
-    return cudaErrorInvalidValue;
+    if (gather != G_PULL) return cudaErrorInvalidValue;
+    if constexpr (!std::is_same<S, double>::value && !TRT) {
+      // more blocks than three per SM; whole gradient, per step: 256x128x128 FP32 368 -> 345
+      // us, 128x64x64 FP32 52.7 -> 49.4, FP16 49.5 -> 46.2, with dforce 65.2 -> 61.2,
+      // 64x40x48 (480 blocks) 23.3 -> 22.5; 48x40x36 with dforce (360 blocks) 18.0 at 80
+      // registers, 19.2 at 64
+      if (g.blocks() > 3 * (int64_t)h.sms)
+        return launch_step(k_adjoint<L, S, G_PULL, TRT, 4>, g.grid, g.block, 0, h.stream, params(h), st, li, lo,
+                           dgamma, dforce, partials);
+    }
+    return launch_step(k_adjoint<L, S, G_PULL, TRT, 0>, g.grid, g.block, 0, h.stream, params(h), st, li, lo, dgamma,
+                       dforce, partials);
   }
   static cudaError_t adjoint(const HostParams& h, int gather, const void* state,
                              const void* lam_in, void* lam_out, double* dgamma, double* dforce,
